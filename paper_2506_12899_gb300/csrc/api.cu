@@ -83,7 +83,8 @@ struct Mlp {
   float* G = nullptr;                // gradients
   float* Am = nullptr;               // Adam first moments
   float* Av = nullptr;               // Adam second moments
-  __nv_bfloat16* Pb = nullptr;       // BF16 copy of the parameters
+  int Hp = 0, Op = 0;                // H and O rounded up to 32 (row lengths of the BF16 copies)
+  __nv_bfloat16* Wb = nullptr;       // the BF16 weight copies (MlpWeights)
   int adam_t = 0;
   int gemm = 0;                      // 0: tcgen05 tensor cores (tc_gemm.cu), 1: warp-level mma.sync
   size_t cap = 0, count = 0;         // training set rows
@@ -114,9 +115,55 @@ struct Mlp {
         return;
       }
   }
-  const __nv_bfloat16* W1b() const { return Pb + oW1; }
-  const __nv_bfloat16* W2b() const { return Pb + oW2; }
-  const __nv_bfloat16* W3b() const { return Pb + oW3; }
+  size_t weight_elems() const { return (size_t)Fpad * Hp + (size_t)Hp * Hp + (size_t)Hp * Op; }
+  const __nv_bfloat16* W1b() const { return Wb; }
+  const __nv_bfloat16* W2b() const { return Wb + (size_t)Fpad * Hp; }
+  const __nv_bfloat16* W3b() const { return W2b() + (size_t)Hp * Hp; }
+  // (the copies as core matrices follow the row-major ones)
+  MlpWeights weights() const {
+    MlpWeights M{};
+    size_t o = 0;
+    const size_t n[3] = {(size_t)Fpad * Hp, (size_t)Hp * Hp, (size_t)Hp * Op};
+    for (int l = 0; l < 3; o += n[l++]) {
+      M.W[l] = Wb + o;
+      M.T[l] = Wb + weight_elems() + o;
+    }
+    M.H = H;
+    M.O = O;
+    M.Hp = Hp;
+    M.Op = Op;
+    M.ob1 = (int)ob1;
+    M.oW2 = (int)oW2;
+    M.ob2 = (int)ob2;
+    M.oW3 = (int)oW3;
+    M.ob3 = (int)ob3;
+    return M;
+  }
+  // The one-launch kernel computes the layers (tcgen05 backend, hidden widths that fit an SM).
+  bool fused() const { return gemm == 0 && mlp_fused_fits(Hp, Op); }
+  MlpTile tile(int rows, const float* Xf, const __nv_bfloat16* X, float* Yout, int early) const {
+    MlpTile T{};
+    T.rows = rows;
+    T.F = F;
+    T.Fpad = Fpad;
+    T.H = H;
+    T.O = O;
+    T.Hp = Hp;
+    T.Op = Op;
+    T.early = early;
+    T.y_vec = reinterpret_cast<uintptr_t>(Yout) % 16 == 0;
+    T.Xf = Xf;
+    T.Xb = X;
+    const MlpWeights M = weights();
+    T.W1 = M.T[0];
+    T.W2 = M.T[1];
+    T.W3 = M.T[2];
+    T.b1 = P + ob1;
+    T.b2 = P + ob2;
+    T.b3 = P + ob3;
+    T.Y = Yout;
+    return T;
+  }
   void ensure_batch(int B) {
     if (B <= bcap) return;
     for (void* q : {(void*)Xb, (void*)H1, (void*)H2, (void*)dYb, (void*)dZ2b, (void*)dZ1b, (void*)Tb, (void*)Y,
@@ -157,9 +204,9 @@ struct Mlp {
   // Yout[rows][O] = MLP(X) with the BF16 weights, hidden activations into h1, h2 ([rows][H]).
   void forward(const __nv_bfloat16* X, int rows, float* Yout, __nv_bfloat16* h1, __nv_bfloat16* h2,
                cudaStream_t st) const {
-    CUDA_TRY(gemm_bf16(gemm, rows, H, Fpad, 0, 0, X, Fpad, W1b(), H, P + ob1, 1, nullptr, h1, H, st));
-    CUDA_TRY(gemm_bf16(gemm, rows, H, H, 0, 0, h1, H, W2b(), H, P + ob2, 1, nullptr, h2, H, st));
-    CUDA_TRY(gemm_bf16(gemm, rows, O, H, 0, 0, h2, H, W3b(), O, P + ob3, 0, Yout, nullptr, O, st));
+    CUDA_TRY(gemm_bf16(gemm, rows, H, Fpad, 0, 0, X, Fpad, W1b(), Hp, P + ob1, 1, nullptr, h1, H, st));
+    CUDA_TRY(gemm_bf16(gemm, rows, H, H, 0, 0, h1, H, W2b(), Hp, P + ob2, 1, nullptr, h2, H, st));
+    CUDA_TRY(gemm_bf16(gemm, rows, O, H, 0, 0, h2, H, W3b(), Op, P + ob3, 0, Yout, nullptr, O, st));
   }
   // G = gradient of the mean squared error over the rows of (X, T), after forward(X, rows, Y,
   // H1, H2); loss_part receives per-block partial sums of the squared errors.
@@ -167,11 +214,11 @@ struct Mlp {
     CUDA_TRY(launch_mse_grad(rows, O, Y, T, dYf, dYb, 1.0f / ((float)rows * O), loss_part, 152, s));
     CUDA_TRY(gemm_bf16(gemm, H, O, rows, 1, 0, H2, H, dYb, O, nullptr, 0, G + oW3, nullptr, O, s));
     CUDA_TRY(launch_colsum(rows, O, dYf, G + ob3, s));
-    CUDA_TRY(gemm_bf16(gemm, rows, H, O, 0, 1, dYb, O, W3b(), O, nullptr, 0, dH2, nullptr, H, s));
+    CUDA_TRY(gemm_bf16(gemm, rows, H, O, 0, 1, dYb, O, W3b(), Op, nullptr, 0, dH2, nullptr, H, s));
     CUDA_TRY(launch_relu_mask(rows * H, dH2, H2, dZ2b, s));
     CUDA_TRY(gemm_bf16(gemm, H, H, rows, 1, 0, H1, H, dZ2b, H, nullptr, 0, G + oW2, nullptr, H, s));
     CUDA_TRY(launch_colsum(rows, H, dH2, G + ob2, s));
-    CUDA_TRY(gemm_bf16(gemm, rows, H, H, 0, 1, dZ2b, H, W2b(), H, nullptr, 0, dH1, nullptr, H, s));
+    CUDA_TRY(gemm_bf16(gemm, rows, H, H, 0, 1, dZ2b, H, W2b(), Hp, nullptr, 0, dH1, nullptr, H, s));
     CUDA_TRY(launch_relu_mask(rows * H, dH1, H1, dZ1b, s));
     CUDA_TRY(gemm_bf16(gemm, Fpad, H, rows, 1, 0, X, Fpad, dZ1b, H, nullptr, 0, G + oW1, nullptr, H, s));
     CUDA_TRY(launch_colsum(rows, H, dH1, G + ob1, s));
@@ -743,7 +790,8 @@ void apply_learned(Context& C, DevLevel& L, const R* r, R* z, cudaStream_t s) {
   const int nb = C.lf_nb;
   CUDA_TRY(launch_mlp_features<R>(nb, C.lf_npatch, L.H.np, C.lf_nstat, C.lf_Fpad, C.mlp_patch, C.mlp_stat, res,
                                   C.mlp_X, C.mlp_s, s));
-  M.forward(C.mlp_X, nb, C.mlp_Y, C.mlp_H1, C.mlp_H2, s);
+  if (M.fused()) CUDA_TRY(launch_mlp_fused(M.tile(nb, nullptr, C.mlp_X, C.mlp_Y, 1), s));
+  else M.forward(C.mlp_X, nb, C.mlp_Y, C.mlp_H1, C.mlp_H2, s);
   // the network predicts the correction in units of s h^(2-d) (A scales like h^(d-2))
   const float hs = (float)std::pow(L.H.h, 2 - L.H.dim);
   CUDA_TRY(launch_mlp_scatter<R>(nb, M.np, M.O, C.mlp_cells, C.mlp_Y, C.mlp_s, C.mlp_scale * hs, z, s));
@@ -1230,7 +1278,7 @@ void set_params(Mlp& M, const float* host) {
   std::memcpy(full.data(), host, (size_t)M.F * M.H * sizeof(float));
   std::memcpy(full.data() + M.ob1, host + (size_t)M.F * M.H, (M.nparam - M.ob1) * sizeof(float));
   CUDA_TRY(cudaMemcpy(M.P, full.data(), M.nparam * sizeof(float), cudaMemcpyHostToDevice));
-  CUDA_TRY(launch_to_bf16((int)M.nparam, M.P, M.Pb, M.s));
+  CUDA_TRY(launch_to_bf16((int)M.nparam, M.P, M.weights(), M.s));
   CUDA_TRY(cudaMemsetAsync(M.Am, 0, M.nparam * sizeof(float), M.s));
   CUDA_TRY(cudaMemsetAsync(M.Av, 0, M.nparam * sizeof(float), M.s));
   CUDA_TRY(cudaStreamSynchronize(M.s));
@@ -1677,6 +1725,8 @@ int sbm_mlp_create(int dim, int p, int hidden, unsigned long long seed, void* st
     M->Fpad = (M->F + 31) / 32 * 32;
     M->H = hidden;
     M->O = M->np;
+    M->Hp = (M->H + 31) / 32 * 32;
+    M->Op = (M->O + 31) / 32 * 32;
     M->s = static_cast<cudaStream_t>(stream);
     const size_t F = M->Fpad, H = M->H, O = M->O;
     M->oW1 = 0;
@@ -1690,7 +1740,8 @@ int sbm_mlp_create(int dim, int p, int hidden, unsigned long long seed, void* st
     M->G = M->alloc<float>(M->nparam);
     M->Am = M->alloc<float>(M->nparam);
     M->Av = M->alloc<float>(M->nparam);
-    M->Pb = M->alloc<__nv_bfloat16>(M->nparam);
+    M->Wb = M->alloc<__nv_bfloat16>(2 * M->weight_elems());
+    CUDA_TRY(cudaMemset(M->Wb, 0, 2 * M->weight_elems() * sizeof(__nv_bfloat16)));
     M->loss_part = M->alloc<float>(152);
     M->loss_tmp = M->alloc<float>(1);
     M->loss_acc = M->alloc<float>(1);
@@ -1751,6 +1802,10 @@ int sbm_mlp_forward(void* mlp, const float* X_dev, int rows, float* Y_dev) {
   Mlp* M = mlp_of(mlp);
   if (!M || !X_dev || !Y_dev || rows < 0) return set_error(SBM_ERR_ARG, "bad argument");
   return guarded([&]() -> int {
+    if (M->fused()) {
+      CUDA_TRY(launch_mlp_fused(M->tile(rows, X_dev, nullptr, Y_dev, 0), M->s));
+      return SBM_OK;
+    }
     M->ensure_batch(std::max(rows, 1));
     CUDA_TRY(launch_pack_bf16(rows, M->F, M->Fpad, X_dev, M->Xb, M->s));
     M->forward(M->Xb, rows, Y_dev, M->H1, M->H2, M->s);
@@ -1812,7 +1867,7 @@ int sbm_mlp_train(void* mlp, int epochs, int batch, float lr, unsigned long long
         M->forward(M->Xb, rows, M->Y, M->H1, M->H2, M->s);
         M->backward(M->Xb, M->Tb, rows);
         M->adam_t += 1;
-        CUDA_TRY(launch_adam((int)M->nparam, M->P, M->G, M->Am, M->Av, M->Pb, lr, 0.9f, 0.999f, 1e-8f, M->adam_t, M->s));
+        CUDA_TRY(launch_adam((int)M->nparam, M->P, M->G, M->Am, M->Av, M->weights(), lr, 0.9f, 0.999f, 1e-8f, M->adam_t, M->s));
         CUDA_TRY(launch_colsum(152, 1, M->loss_part, M->loss_tmp, M->s));
         CUDA_TRY(launch_axpy_f(1, 1.0f / ((float)rows * M->O), M->loss_tmp, M->loss_acc, M->s));
         ++nbatch;

@@ -30,6 +30,7 @@ __global__ void __launch_bounds__(256) k_mlp_features(int n_bnd, int npatch, int
                                                       float* __restrict__ s_out) {
   const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  pdl_entry();
   if (b >= n_bnd) return;
   const int nv = npatch * np;
   float ss = 0.f;
@@ -190,9 +191,26 @@ __global__ void k_colsum(int rows, int cols, const float* __restrict__ D, float*
   }
 }
 
+// Parameter e of the packed vector rounded into the two BF16 copies (biases have none).
+__device__ __forceinline__ void store_weight(const MlpWeights& M, int e, float w) {
+  int l, i, o, ld;                                   // matrix, input, output, row length
+  if (e < M.ob1) {
+    l = 0, i = e / M.H, o = e % M.H, ld = M.Hp;
+  } else if (e >= M.oW2 && e < M.ob2) {
+    l = 1, i = (e - M.oW2) / M.H, o = (e - M.oW2) % M.H, ld = M.Hp;
+  } else if (e >= M.oW3 && e < M.ob3) {
+    l = 2, i = (e - M.oW3) / M.O, o = (e - M.oW3) % M.O, ld = M.Op;
+  } else {
+    return;
+  }
+  const __nv_bfloat16 b = __float2bfloat16_rn(w);
+  M.W[l][(size_t)i * ld + o] = b;
+  M.T[l][((size_t)(i >> 3) * (ld >> 3) + (o >> 3)) * 64 + (i & 7) * 8 + (o & 7)] = b;
+}
+
 // Adam (Kingma & Ba) on FP32 master parameters; writes the BF16 copy used by the forward pass.
 __global__ void k_adam(int n, float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                       float* __restrict__ v, __nv_bfloat16* __restrict__ pb, float lr, float b1, float b2, float eps,
+                       float* __restrict__ v, const __grid_constant__ MlpWeights W, float lr, float b1, float b2, float eps,
                        float c1, float c2) {
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
     const float gg = g[e];
@@ -202,13 +220,12 @@ __global__ void k_adam(int n, float* __restrict__ p, const float* __restrict__ g
     v[e] = vv;
     const float w = p[e] - lr * (mm / c1) / (sqrtf(vv / c2) + eps);
     p[e] = w;
-    if (pb) pb[e] = __float2bfloat16_rn(w);
+    store_weight(W, e, w);
   }
 }
 
-__global__ void k_to_bf16(int n, const float* __restrict__ x, __nv_bfloat16* __restrict__ y) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x)
-    y[e] = __float2bfloat16_rn(x[e]);
+__global__ void k_to_bf16(int n, const float* __restrict__ x, const __grid_constant__ MlpWeights W) {
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) store_weight(W, e, x[e]);
 }
 
 // T[b][i] = -u[cell(b)][i] / s[b]  (training target: the error of u for the zero solution).
@@ -252,6 +269,7 @@ __global__ void k_scale_f(size_t n, float a, float* __restrict__ x) {
 template <typename TZ>
 __global__ void k_mlp_scatter(int n_bnd, int np, int ldy, const int* __restrict__ cell, const float* __restrict__ Y,
                               const float* __restrict__ s, float scale, TZ* __restrict__ z) {
+  pdl_entry();
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n_bnd * np; e += gridDim.x * blockDim.x) {
     const int b = e / np, i = e % np;
     z[(size_t)cell[b] * np + i] += (TZ)(scale * s[b] * Y[(size_t)b * ldy + i]);
@@ -323,7 +341,7 @@ template <typename TI>
 cudaError_t launch_mlp_features(int n_bnd, int npatch, int np, int nstat, int Fpad, const int* patch,
                                 const float* stat, const TI* res, __nv_bfloat16* X, float* s, cudaStream_t st) {
   if (n_bnd == 0) return cudaSuccess;
-  k_mlp_features<TI><<<(n_bnd + 7) / 8, 256, 0, st>>>(n_bnd, npatch, np, nstat, Fpad, patch, stat, res, X, s);
+  SBM_PDL((k_mlp_features<TI>), (n_bnd + 7) / 8, 256, 0, st, n_bnd, npatch, np, nstat, Fpad, patch, stat, res, X, s);
   count_launches();
   return cudaGetLastError();
 }
@@ -360,16 +378,16 @@ cudaError_t launch_colsum(int rows, int cols, const float* D, float* g, cudaStre
   return cudaGetLastError();
 }
 
-cudaError_t launch_adam(int n, float* p, const float* g, float* m, float* v, __nv_bfloat16* pb, float lr, float b1,
+cudaError_t launch_adam(int n, float* p, const float* g, float* m, float* v, const MlpWeights& W, float lr, float b1,
                         float b2, float eps, int t, cudaStream_t s) {
   const float c1 = 1.f - powf(b1, (float)t), c2 = 1.f - powf(b2, (float)t);
-  k_adam<<<g1(n), 256, 0, s>>>(n, p, g, m, v, pb, lr, b1, b2, eps, c1, c2);
+  k_adam<<<g1(n), 256, 0, s>>>(n, p, g, m, v, W, lr, b1, b2, eps, c1, c2);
   count_launches();
   return cudaGetLastError();
 }
 
-cudaError_t launch_to_bf16(int n, const float* x, __nv_bfloat16* y, cudaStream_t s) {
-  k_to_bf16<<<g1(n), 256, 0, s>>>(n, x, y);
+cudaError_t launch_to_bf16(int n, const float* x, const MlpWeights& W, cudaStream_t s) {
+  k_to_bf16<<<g1(n), 256, 0, s>>>(n, x, W);
   count_launches();
   return cudaGetLastError();
 }
@@ -385,7 +403,7 @@ cudaError_t launch_mlp_targets(int n_bnd, int np, const int* cell, const TU* u, 
 template <typename TZ>
 cudaError_t launch_mlp_scatter(int n_bnd, int np, int ldy, const int* cell, const float* Y, const float* s,
                                float scale, TZ* z, cudaStream_t st) {
-  k_mlp_scatter<TZ><<<g1(n_bnd * np), 256, 0, st>>>(n_bnd, np, ldy, cell, Y, s, scale, z);
+  SBM_PDL((k_mlp_scatter<TZ>), g1(n_bnd * np), 256, 0, st, n_bnd, np, ldy, cell, Y, s, scale, z);
   count_launches();
   return cudaGetLastError();
 }

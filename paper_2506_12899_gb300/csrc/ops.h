@@ -383,13 +383,38 @@ cudaError_t launch_gemm_tc(int M, int N, int K, int ta, int tb, const __nv_bfloa
                            const __nv_bfloat16* B, int ldb, const float* bias, int relu, float* Cf,
                            __nv_bfloat16* Cb, int ldc, cudaStream_t s);
 int tc_fault_take();
+// The whole MLP over one batch of rows in one launch (tc_gemm.cu), for hidden widths that
+// mlp_fused_fits: Y = W3^T relu(W2^T relu(W1^T x + b1) + b2) + b3 for every row x.  Xf: FP32 rows of F
+// features, or (Xf null) Xb: BF16 rows of Fpad.  W1, W2, W3: the core-matrix copies of the weights
+// (MlpWeights); Hp and Op are H and O rounded up to 32.
+// early: the weights were written two or more launches back (they are read before the
+// dependency wait).
+struct MlpTile {
+  int rows, F, Fpad, H, O, Hp, Op, early;
+  bool y_vec;                      // Y is 16-byte aligned
+  const float* Xf;
+  const __nv_bfloat16 *Xb, *W1, *W2, *W3;
+  const float *b1, *b2, *b3;
+  float* Y;
+};
+bool mlp_fused_fits(int Hp, int Op);
+cudaError_t launch_mlp_fused(const MlpTile& P, cudaStream_t s);
+// The BF16 copies of the weight matrices W1 [Fpad][Hp], W2 [Hp][Hp], W3 [Hp][Op] (inputs x outputs,
+// zero in the padding): W row-major, T as core matrices of 8 inputs x 8 outputs (128 bytes, outputs
+// contiguous), those of one group of inputs side by side; and where each matrix and bias starts
+// in the packed FP32 parameter vector (W1 first).
+struct MlpWeights {
+  __nv_bfloat16 *W[3], *T[3];
+  int H, O, Hp, Op, ob1, oW2, ob2, oW3, ob3;
+};
 cudaError_t launch_mse_grad(int rows, int O, const float* Y, const float* T, float* dYf, __nv_bfloat16* dYb,
                             float inv_count, float* loss_partial, int nblk, cudaStream_t s);
 cudaError_t launch_relu_mask(int n, float* dH, const __nv_bfloat16* H, __nv_bfloat16* dZb, cudaStream_t s);
 cudaError_t launch_colsum(int rows, int cols, const float* D, float* g, cudaStream_t s);
-cudaError_t launch_adam(int n, float* p, const float* g, float* m, float* v, __nv_bfloat16* pb, float lr, float b1,
+cudaError_t launch_adam(int n, float* p, const float* g, float* m, float* v, const MlpWeights& W, float lr, float b1,
                         float b2, float eps, int t, cudaStream_t s);
-cudaError_t launch_to_bf16(int n, const float* x, __nv_bfloat16* y, cudaStream_t s);
+// BF16 copies of the weight matrices of the packed parameters x.
+cudaError_t launch_to_bf16(int n, const float* x, const MlpWeights& W, cudaStream_t s);
 template <typename TU>
 cudaError_t launch_mlp_targets(int n_bnd, int np, const int* cell, const TU* u, const float* s, float hfac, float* T,
                                cudaStream_t st);

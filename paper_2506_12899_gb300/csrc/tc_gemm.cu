@@ -14,6 +14,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "ops.h"
@@ -21,23 +22,12 @@
 namespace sbm {
 namespace {
 
+#include "tc_core.cuh"
+
 constexpr int TBM = 128, TBN = 128, TBK = 64;
 constexpr int kTcThreads = 128;
 
 __device__ int g_tc_fault = 0;
-
-// Shared-memory matrix descriptor (tcgen05): start address, leading (K direction) and stride
-// (8-row groups) byte offsets, all >> 4; bits 46-48 hold the fixed value 1; no swizzle.
-__device__ __forceinline__ uint64_t smem_desc(const void* p, uint32_t lbo, uint32_t sbo) {
-  const uint64_t a = (uint64_t)(smem_addr(p) >> 4) & 0x3FFFu;
-  return a | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) | ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
-}
-
-// Instruction descriptor of tcgen05.mma kind::f16: FP32 accumulator, BF16 A and B, both K-major,
-// N >> 3 and M >> 4.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
 
 // Byte offset of element (row r, k) of a 128 x 64 K-major no-swizzle tile.
 __device__ __forceinline__ uint32_t tile_off(int r, int k) {
@@ -149,8 +139,8 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_tc(int M, int N, int K, con
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
       for (int ks = 0; ks < TBK / 16; ++ks) {        // K = 16 per instruction: two core matrices
-        const uint64_t ad = smem_desc(As + ks * 256, 128, 1024);
-        const uint64_t bd = smem_desc(Bs + ks * 256, 128, 1024);
+        const uint64_t ad = smem_desc(smem_addr(As + ks * 256), 128, 1024);
+        const uint64_t bd = smem_desc(smem_addr(Bs + ks * 256), 128, 1024);
         const uint32_t acc = (it > 0 || ks > 0) ? 1u : 0u;
         asm volatile(
             "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
@@ -224,6 +214,273 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_tc(int M, int N, int K, con
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(tmem) : "memory");
 }
 
+// ----------------------------------------------------------------------------------------------
+// The learned correction's MLP, F -> H -> H -> O, as one kernel on the tcgen05 tensor cores.
+//
+// A CTA takes a tile of 128 rows through all layers: the first layer streams the features and W1 in
+// chunks of 64 features, the accumulator (128 x H FP32) stays in tensor memory, the activations
+// go through registers (bias, ReLU, BF16) into a shared-memory tile that is the next layer's A
+// operand, and only the outputs reach global memory.  Three roles run apart from one another,
+// joined by mbarriers (in one loop of all threads, the feature loads, the weight copies and the
+// tensor core's latency added up: 55 us against 40 at 16,384 x 2023 -> 128 -> 128 -> 64; four launches,
+// the rounding of X among them, took 432):
+//   - 16 warps bring the features of the first layer into a ring of A tiles and carry out the
+//     epilogues;
+//   - one thread copies the weight chunks of all layers, one after the other, into a ring of B
+//     tiles; the weights are stored as core matrices, so a chunk is one contiguous bulk copy, and
+//     the next layer's weights are in flight while a layer ends;
+//   - one thread issues the MMAs.
+// FP32 features are rounded to BF16 on the way in: a thread loads eight rows of one feature (each
+// load instruction of a warp reads 32 consecutive features of a row, whatever the row's alignment)
+// and writes them as one 16-byte piece of an MN-major operand, three chunks ahead in registers.
+//
+// What bounds it: with FP32 features the read of X (16,384 x 2023: 133 MB, 19.5 us at the measured
+// copy bandwidth; 128 of the 152 SMs have a tile, each with three chunks of 32 KB in flight); with few
+// rows the chain of layers (260 rows x 192: three GEMM launches took 97 us of a V-cycle, now 17).
+constexpr int kTileRows = 128;
+constexpr int kFeedWarps = 16;                     // feature loads and epilogues
+constexpr int kFusedThreads = (kFeedWarps + 2) * 32;
+
+// SA, SB: stages of the A and B rings.  F32IN: X is FP32 [rows][F], else BF16 [rows][Fpad].
+template <int SA, int SB, bool F32IN>
+__global__ void __launch_bounds__(kFusedThreads, 1) k_mlp_fused(const __grid_constant__ MlpTile P) {
+  extern __shared__ __align__(1024) unsigned char fused_smem[];
+  __shared__ __align__(8) unsigned long long full_a[SA], empty_a[SA], full_b[SB], empty_b[SB], acc_full, act_full;
+  __shared__ uint32_t tmem_base;
+  __shared__ int failed;
+  const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+  const int Hp = P.Hp, Op = P.Op, wmax = max(Hp, Op);
+  constexpr uint32_t kABytes = kTileRows * kChunkK * 2;
+  const uint32_t b_bytes = (uint32_t)wmax * kChunkK * 2;
+  const uint32_t ring_a = smem_addr(fused_smem), ring_b = ring_a + SA * kABytes, act = ring_b + SB * b_bytes;
+  const uint32_t act_sbo = (uint32_t)wmax * 16;      // bytes between the 8-row groups of the activation tile
+  const int ntile = (P.rows + kTileRows - 1) / kTileRows;
+  // chunks of the layers, in order
+  const int n1 = (P.Fpad + kChunkK - 1) / kChunkK, n2 = (Hp + kChunkK - 1) / kChunkK;
+  const int total = n1 + 2 * n2;
+  uint32_t ncols = 32;
+  while ((int)ncols < wmax) ncols <<= 1;
+
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_base)),
+                 "r"(ncols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < SA; ++s) {
+      mbar_init(&full_a[s], kFeedWarps);
+      mbar_init(&empty_a[s], 1);
+    }
+    for (int s = 0; s < SB; ++s) {
+      mbar_init(&full_b[s], 1);
+      mbar_init(&empty_b[s], 1);
+    }
+    mbar_init(&acc_full, 1);
+    mbar_init(&act_full, kFeedWarps);
+    mbar_fence_init();
+    failed = 0;
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_base;
+  volatile int* stop = &failed;
+  // a bounded wait; once one has run out, every role leaves its loop
+  auto wait = [&](unsigned long long* bar, unsigned parity) {
+    if (!mbar_wait(bar, parity)) *stop = 1;
+    return *stop == 0;
+  };
+
+  if (warp == kFeedWarps) {                          // the weights
+    if (lane == 0) {
+      if (!P.early) pdl_wait();                      // early: written two or more launches back
+      int g = 0;                                     // chunks of the ring so far
+      bool ok = true;
+      for (int tile = blockIdx.x; tile < ntile && ok; tile += gridDim.x)
+        for (int i = 0; i < total && ok; ++i, ++g) {
+          if (g >= SB) ok = wait(&empty_b[g % SB], (unsigned)((g / SB - 1) & 1));
+          if (!ok) break;
+          const int at = i < n1 ? i : (i < n1 + n2 ? i - n1 : i - n1 - n2);
+          const int K = i < n1 ? P.Fpad : Hp, np = i < n1 + n2 ? Hp : Op;
+          const __nv_bfloat16* W = i < n1 ? P.W1 : (i < n1 + n2 ? P.W2 : P.W3);
+          const unsigned bytes = (unsigned)(min(kChunkK, K - at * kChunkK) * np * 2);
+          mbar_arrive_tx(&full_b[g % SB], bytes);
+          bulk_load(fused_smem + SA * kABytes + (g % SB) * b_bytes, W + (size_t)at * kChunkK * np, bytes, &full_b[g % SB]);
+        }
+    }
+  } else if (warp == kFeedWarps + 1) {               // the tensor core
+    if (lane == 0) {
+      int ga = 0, gb = 0, layers = 0;                // A and B chunks, layers with an activation tile so far
+      bool ok = true;
+      for (int tile = blockIdx.x; tile < ntile && ok; tile += gridDim.x)
+        for (int i = 0; i < total && ok; ++i, ++gb) {
+          const int layer = i < n1 ? 0 : (i < n1 + n2 ? 1 : 2);
+          const int at = i - (layer == 0 ? 0 : (layer == 1 ? n1 : n1 + n2));
+          const int K = layer == 0 ? P.Fpad : Hp, np = layer == 2 ? Op : Hp;
+          if (layer == 0) ok = wait(&full_a[ga % SA], (unsigned)((ga / SA) & 1));
+          else if (at == 0) ok = wait(&act_full, (unsigned)(layers++ & 1));
+          if (layer == 0 && at == 0 && tile != (int)blockIdx.x) ok = wait(&act_full, (unsigned)(layers++ & 1)) && ok;
+          ok = ok && wait(&full_b[gb % SB], (unsigned)((gb / SB) & 1));
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t a = layer == 0 ? ring_a + (ga % SA) * kABytes : act + (uint32_t)at * (kChunkK / 8) * 128;
+          const uint32_t b = ring_b + (gb % SB) * b_bytes;
+          const uint32_t id = idesc_bf16(kTileRows, np, F32IN && layer == 0, true);
+          for (int ks = 0; ks < min(kChunkK, K - at * kChunkK) / 16; ++ks)
+            mma_bf16(tmem, smem_desc(a + ks * 256, 128, layer == 0 ? 1024 : act_sbo),
+                     smem_desc(b + ks * (uint32_t)np * 32, (uint32_t)np * 16, 128), id, at > 0 || ks > 0);
+          if (layer == 0) mma_commit(&empty_a[ga++ % SA]);
+          mma_commit(&empty_b[gb % SB]);
+          if (i == n1 - 1 || i == n1 + n2 - 1 || i == total - 1) mma_commit(&acc_full);
+        }
+    }
+  } else {                                           // features and epilogues
+    pdl_wait();
+    pdl_trigger();
+    int ga = 0, layers = 0;
+    bool ok = true;
+    auto arrive = [&](unsigned long long* bar) {     // this warp's writes to shared memory, then one arrival
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_addr(bar))
+                     : "memory");
+    };
+    auto stage_free = [&](int g) { return g < SA || wait(&empty_a[g % SA], (unsigned)((g / SA - 1) & 1)); };
+    for (int tile = blockIdx.x; tile < ntile && ok; tile += gridDim.x) {
+      const int row0 = tile * kTileRows;
+      if constexpr (F32IN) {
+        // FP32 features of chunk i: features lane and lane + 32 of the warp's 8 rows
+        auto load_x = [&](int i, float (&v)[16]) {
+          const int k = i * kChunkK + lane;
+          const float* src = P.Xf + (size_t)(row0 + 8 * warp) * P.F + k;
+          if (row0 + 8 * warp + 8 <= P.rows && (i + 1) * kChunkK <= P.F) {
+#pragma unroll
+            for (int r = 0; r < 8; ++r, src += P.F) {
+              v[r] = __ldcs(src);
+              v[8 + r] = __ldcs(src + 32);
+            }
+          } else {
+#pragma unroll
+            for (int r = 0; r < 8; ++r, src += P.F) {
+              const bool in = row0 + 8 * warp + r < P.rows;
+              v[r] = in && k < P.F ? __ldcs(src) : 0.f;
+              v[8 + r] = in && k + 32 < P.F ? __ldcs(src + 32) : 0.f;
+            }
+          }
+        };
+        auto put = [&](int i, float (&v)[16]) {      // chunk i into its stage, chunk i + 3 into the registers
+          if (i >= n1 || !ok) return;
+          ok = stage_free(ga);
+          if (!ok) return;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {              // one 16-byte piece (8 rows) per feature
+            uint32_t w[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const __nv_bfloat162 b = __floats2bfloat162_rn(v[8 * h + 2 * q], v[8 * h + 2 * q + 1]);
+              w[q] = *reinterpret_cast<const uint32_t*>(&b);
+            }
+            const int k = lane + 32 * h;
+            asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(ring_a + (ga % SA) * kABytes + warp * 1024 +
+                                                                       (k >> 3) * 128 + (k & 7) * 16),
+                         "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
+                         : "memory");
+          }
+          if (i + 3 < n1) load_x(i + 3, v);
+          arrive(&full_a[ga % SA]);
+          ++ga;
+        };
+        float va[16], vb[16], vc[16];
+        load_x(0, va);
+        if (n1 > 1) load_x(1, vb);
+        if (n1 > 2) load_x(2, vc);
+        for (int i = 0; i < n1 && ok; i += 3) {
+          put(i, va);
+          put(i + 1, vb);
+          put(i + 2, vc);
+        }
+      } else {                                       // BF16 rows, copied asynchronously, two chunks in flight
+        for (int i = 0; i < n1 + 2 && ok; ++i) {
+          if (i < n1) {
+            ok = stage_free(ga + i);
+            if (ok)
+              stage_async<true>(ring_a + ((ga + i) % SA) * kABytes, P.Xb, P.Fpad, P.rows, P.Fpad, row0, kTileRows,
+                                i * kChunkK, (int)threadIdx.x, kFeedWarps * 32);
+          }
+          cp_async_commit();
+          cp_async_wait<2>();
+          if (i >= 2) arrive(&full_a[(ga + i - 2) % SA]);
+        }
+        ga += n1;
+      }
+      // The end of a layer: the accumulator through bias and ReLU into the activation tile, or to
+      // the output.  Four warps share a row quarter and take a quarter of the columns each.
+      for (int layer = 0; layer < 3 && ok; ++layer) {
+        ok = wait(&acc_full, (unsigned)(layers++ & 1));
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const int r = 32 * (warp & 3) + lane, row = row0 + r;
+        const int np = layer == 2 ? Op : Hp, n = layer == 2 ? P.O : P.H;
+        const float* bias = layer == 0 ? P.b1 : (layer == 1 ? P.b2 : P.b3);
+        for (int c0 = (warp >> 2) * (np / 4); c0 < ((warp >> 2) + 1) * (np / 4); c0 += 8) {
+          float v[8];
+          tmem_ld8(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, v);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) v[j] = c0 + j < n ? v[j] + bias[c0 + j] : 0.f;
+          if (layer < 2) {
+            uint32_t w[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const __nv_bfloat162 b = __floats2bfloat162_rn(fmaxf(v[2 * q], 0.f), fmaxf(v[2 * q + 1], 0.f));
+              w[q] = *reinterpret_cast<const uint32_t*>(&b);
+            }
+            asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(act + (uint32_t)(r >> 3) * act_sbo +
+                                                                       (uint32_t)(c0 / 8) * 128 + (r & 7) * 16),
+                         "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
+                         : "memory");
+          } else if (row < P.rows) {
+            float* y = P.Y + (size_t)row * P.O + c0;
+            if ((P.O & 3) == 0 && c0 + 8 <= P.O && P.y_vec) {
+              reinterpret_cast<float4*>(y)[0] = make_float4(v[0], v[1], v[2], v[3]);
+              reinterpret_cast<float4*>(y)[1] = make_float4(v[4], v[5], v[6], v[7]);
+            } else {
+#pragma unroll
+              for (int j = 0; j < 8; ++j)
+                if (c0 + j < P.O) y[j] = v[j];
+            }
+          }
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        arrive(&act_full);                           // the tile is written and the accumulator read
+      }
+    }
+    cp_async_wait<0>();
+  }
+  __syncthreads();
+  if (failed && threadIdx.x == 0) {                  // record it; copies and MMAs in flight get time to land
+    atomicExch(&g_tc_fault, 1);
+    for (int s = 0; s < SB; ++s)
+      for (unsigned p = 0; p < 2; ++p) mbar_wait(&full_b[s], p, 1u << 16);
+    for (unsigned p = 0; p < 2; ++p) mbar_wait(&acc_full, p, 1u << 16);
+  }
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
+}
+
+template <int SA, int SB, bool F32IN>
+cudaError_t launch_fused(const MlpTile& P, size_t smem, cudaStream_t s) {
+  const cudaError_t e = cudaFuncSetAttribute(k_mlp_fused<SA, SB, F32IN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem);
+  if (e != cudaSuccess) return e;
+  const int ntile = (P.rows + kTileRows - 1) / kTileRows;
+  SBM_PDL((k_mlp_fused<SA, SB, F32IN>), (unsigned)std::min(ntile, 152), kFusedThreads, smem, s, P);
+  return cudaSuccess;
+}
+
 }  // namespace
 
 // Two stages of 32 KB: at most 3 CTAs per SM, so the CTAs of an SM never ask for more than 3 x 128
@@ -250,6 +507,24 @@ cudaError_t launch_gemm_tc(int M, int N, int K, int ta, int tb, const __nv_bfloa
   else if (!ta && tb) e = launch_tc<0, 1>(grid, M, N, K, A, lda, B, ldb, bias, relu, Cf, Cb, ldc, s);
   else if (ta && !tb) e = launch_tc<1, 0>(grid, M, N, K, A, lda, B, ldb, bias, relu, Cf, Cb, ldc, s);
   else e = launch_tc<1, 1>(grid, M, N, K, A, lda, B, ldb, bias, relu, Cf, Cb, ldc, s);
+  if (e != cudaSuccess) return e;
+  count_launches();
+  return cudaGetLastError();
+}
+
+// Hidden widths up to 256: four A stages, three B stages of 64 x 256 BF16 and the 128 x 256 activation
+// tile (224 KB) still fit an SM; wider networks run layer by layer.
+bool mlp_fused_fits(int Hp, int Op) { return std::max(Hp, Op) <= 256; }
+
+cudaError_t launch_mlp_fused(const MlpTile& P, cudaStream_t s) {
+  if (P.rows == 0) return cudaSuccess;
+  const size_t w = (size_t)std::max(P.Hp, P.Op);
+  const size_t a = kTileRows * kChunkK * 2, b = w * kChunkK * 2, act = kTileRows * w * 2;
+  cudaError_t e;
+  if (w <= 128)
+    e = P.Xf ? launch_fused<5, 5, true>(P, 5 * a + 5 * b + act, s) : launch_fused<5, 5, false>(P, 5 * a + 5 * b + act, s);
+  else
+    e = P.Xf ? launch_fused<4, 3, true>(P, 4 * a + 3 * b + act, s) : launch_fused<4, 3, false>(P, 4 * a + 3 * b + act, s);
   if (e != cudaSuccess) return e;
   count_launches();
   return cudaGetLastError();

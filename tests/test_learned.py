@@ -240,3 +240,19 @@ def test_tensor_core_gemm_matches_mma_sync(dim, p, hidden, rows):
     assert np.linalg.norm(y_tc - y_ws) <= 1e-4 * np.linalg.norm(y_ws)
     assert abs(l_tc - l_ws) <= 1e-4 * l_ws
     assert np.linalg.norm(g_tc - g_ws) <= 1e-3 * np.linalg.norm(g_ws)
+
+
+@pytest.mark.parametrize("dim,p,hidden,rows", [(2, 1, 8, 1), (2, 2, 33, 127), (3, 1, 128, 128), (2, 3, 200, 129),
+                                               (3, 2, 256, 300), (2, 1, 264, 140), (2, 1, 32, 152 * 128 + 5)])
+def test_forward_edges_match_mma_sync(dim, p, hidden, rows):
+    """The one-launch forward pass (hidden widths up to 256) and the layer-by-layer one (264) against the
+    mma.sync layers at the edges of the 128-row tiles, of the padded widths, and past one tile per SM.
+    Same BF16 products, FP32 sums in another order: an activation next to a rounding boundary may round
+    the other way, one BF16 unit (2^-8) of one hidden value."""
+    import paper_2506_12899_gb300 as S
+    gm = S.Mlp(dim, p, hidden, seed=3)
+    X = torch.rand((rows, gm.F), generator=torch.Generator(device="cuda").manual_seed(rows), device="cuda") * 2 - 1
+    y = gm.forward(X)
+    gm.gemm_backend(1)
+    ref = gm.forward(X)
+    assert torch.isfinite(y).all() and (y - ref).norm() <= 2.0 ** -8 * ref.norm()
