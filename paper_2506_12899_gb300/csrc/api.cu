@@ -95,6 +95,8 @@ struct Mlp {
   __nv_bfloat16 *Xb = nullptr, *H1 = nullptr, *H2 = nullptr, *dYb = nullptr, *dZ2b = nullptr, *dZ1b = nullptr;
   float *Tb = nullptr, *Y = nullptr, *dYf = nullptr, *dH2 = nullptr, *dH1 = nullptr, *loss_part = nullptr,
         *loss_tmp = nullptr, *loss_acc = nullptr;
+  float *grad_part = nullptr, *bias_part = nullptr;   // partial sums of the one-launch training pass
+  size_t grad_part_len = 0;
   ~Mlp() {
     for (void* q : allocs) cudaFree(q);
   }
@@ -169,12 +171,12 @@ struct Mlp {
     for (void* q : {(void*)Xb, (void*)H1, (void*)H2, (void*)dYb, (void*)dZ2b, (void*)dZ1b, (void*)Tb, (void*)Y,
                     (void*)dYf, (void*)dH2, (void*)dH1})
       release(q);
-    Xb = alloc<__nv_bfloat16>((size_t)B * Fpad);
-    H1 = alloc<__nv_bfloat16>((size_t)B * H);
-    H2 = alloc<__nv_bfloat16>((size_t)B * H);
-    dYb = alloc<__nv_bfloat16>((size_t)B * O);
-    dZ2b = alloc<__nv_bfloat16>((size_t)B * H);
-    dZ1b = alloc<__nv_bfloat16>((size_t)B * H);
+    Xb = alloc<__nv_bfloat16>((size_t)B * Fpad);     // (rows of the one-launch pass are padded to Hp, Op)
+    H1 = alloc<__nv_bfloat16>((size_t)B * Hp);
+    H2 = alloc<__nv_bfloat16>((size_t)B * Hp);
+    dYb = alloc<__nv_bfloat16>((size_t)B * Op);
+    dZ2b = alloc<__nv_bfloat16>((size_t)B * Hp);
+    dZ1b = alloc<__nv_bfloat16>((size_t)B * Hp);
     Tb = alloc<float>((size_t)B * O);
     Y = alloc<float>((size_t)B * O);
     dYf = alloc<float>((size_t)B * O);
@@ -207,6 +209,50 @@ struct Mlp {
     CUDA_TRY(gemm_bf16(gemm, rows, H, Fpad, 0, 0, X, Fpad, W1b(), Hp, P + ob1, 1, nullptr, h1, H, st));
     CUDA_TRY(gemm_bf16(gemm, rows, H, H, 0, 0, h1, H, W2b(), Hp, P + ob2, 1, nullptr, h2, H, st));
     CUDA_TRY(gemm_bf16(gemm, rows, O, H, 0, 0, h2, H, W3b(), Op, P + ob3, 0, Yout, nullptr, O, st));
+  }
+  // G = gradient of the mean squared error over the rows of (X, T), X FP32 (Xf) or BF16 in the batch
+  // buffer Xb (Xf null); loss_part receives partial sums of the squared errors.
+  void train_pass(const float* Xf, const float* T, int rows) {
+    if (!fused()) {
+      if (Xf) CUDA_TRY(launch_pack_bf16(rows, F, Fpad, Xf, Xb, s));
+      forward(Xb, rows, Y, H1, H2, s);
+      backward(Xb, T, rows);
+      return;
+    }
+    WgradArgs A{};
+    const int mh = (H + 127) / 128, mf = (Fpad + 127) / 128, mo = (O + 127) / 128;
+    A.g[0] = {Xb, dZ1b, Fpad, Fpad, Hp, H, mf, mh, oW1};
+    A.g[1] = {H1, dZ2b, Hp, H, Hp, H, mh, mh, oW2};
+    A.g[2] = {H2, dYb, Hp, H, Op, O, mh, mo, oW3};
+    // as many row ranges as give every SM one tile, none shorter than 128 rows
+    const int tiles = mf * mh + mh * mh + mh * mo;
+    const int want = std::max(1, std::min(152 / tiles, (rows + 127) / 128));
+    A.split_rows = ((rows + want - 1) / want + 63) / 64 * 64;
+    A.splits = (rows + A.split_rows - 1) / A.split_rows;
+    A.rows = rows;
+    A.part_stride = (nparam + 3) / 4 * 4;
+    if (grad_part_len < A.splits * A.part_stride) {
+      release(grad_part);
+      grad_part = nullptr;
+      grad_part_len = 0;
+      grad_part = alloc<float>(A.splits * A.part_stride);
+      grad_part_len = A.splits * A.part_stride;
+    }
+    if (!bias_part) bias_part = alloc<float>((size_t)kLossParts * (2 * Hp + Op));
+    A.part = grad_part;
+    MlpTile t = tile(rows, Xf, Xf ? nullptr : Xb, nullptr, 0);
+    t.T = T;
+    t.inv_count = 1.0f / ((float)rows * O);
+    t.Xs = Xb;
+    t.H1 = H1;
+    t.H2 = H2;
+    t.dY = dYb;
+    t.dZ2 = dZ2b;
+    t.dZ1 = dZ1b;
+    t.bias_part = bias_part;
+    t.loss_part = loss_part;
+    CUDA_TRY(launch_mlp_fused(t, s));
+    CUDA_TRY(launch_wgrad(A, (int)nparam, mlp_fused_ctas(rows), bias_part, weights(), G, s));
   }
   // G = gradient of the mean squared error over the rows of (X, T), after forward(X, rows, Y,
   // H1, H2); loss_part receives per-block partial sums of the squared errors.
@@ -1286,10 +1332,8 @@ void set_params(Mlp& M, const float* host) {
 }
 
 void get_packed(const Mlp& M, const float* dev, float* host) {
-  std::vector<float> full(M.nparam);
-  CUDA_TRY(cudaMemcpy(full.data(), dev, M.nparam * sizeof(float), cudaMemcpyDeviceToHost));
-  std::memcpy(host, full.data(), (size_t)M.F * M.H * sizeof(float));
-  std::memcpy(host + (size_t)M.F * M.H, full.data() + M.ob1, (M.nparam - M.ob1) * sizeof(float));
+  CUDA_TRY(cudaMemcpy(host, dev, (size_t)M.F * M.H * sizeof(float), cudaMemcpyDeviceToHost));
+  CUDA_TRY(cudaMemcpy(host + (size_t)M.F * M.H, dev + M.ob1, (M.nparam - M.ob1) * sizeof(float), cudaMemcpyDeviceToHost));
 }
 
 // Sum of the squared-error partials of the last backward pass, on the host.
@@ -1742,7 +1786,7 @@ int sbm_mlp_create(int dim, int p, int hidden, unsigned long long seed, void* st
     M->Av = M->alloc<float>(M->nparam);
     M->Wb = M->alloc<__nv_bfloat16>(2 * M->weight_elems());
     CUDA_TRY(cudaMemset(M->Wb, 0, 2 * M->weight_elems() * sizeof(__nv_bfloat16)));
-    M->loss_part = M->alloc<float>(152);
+    M->loss_part = M->alloc<float>(kLossParts);
     M->loss_tmp = M->alloc<float>(1);
     M->loss_acc = M->alloc<float>(1);
     // He-normal hidden layers, 1/H output layer, zero biases
@@ -1819,10 +1863,7 @@ int sbm_mlp_gradients(void* mlp, const float* X_dev, const float* T_dev, int row
   if (!M || !X_dev || !T_dev || rows < 1) return set_error(SBM_ERR_ARG, "bad argument");
   return guarded([&]() -> int {
     M->ensure_batch(rows);
-    CUDA_TRY(launch_pack_bf16(rows, M->F, M->Fpad, X_dev, M->Xb, M->s));
-    CUDA_TRY(cudaMemcpyAsync(M->Tb, T_dev, (size_t)rows * M->O * sizeof(float), cudaMemcpyDeviceToDevice, M->s));
-    M->forward(M->Xb, rows, M->Y, M->H1, M->H2, M->s);
-    M->backward(M->Xb, M->Tb, rows);
+    M->train_pass(X_dev, T_dev, rows);
     const double l = read_loss(*M, rows);
     if (tc_fault_take() != 0) return set_error(SBM_ERR_CUDA, "a tensor-core GEMM commit did not arrive in time");
     if (loss) *loss = l;
@@ -1864,8 +1905,7 @@ int sbm_mlp_train(void* mlp, int epochs, int batch, float lr, unsigned long long
       for (size_t b0 = 0; b0 < n; b0 += batch) {
         const int rows = (int)std::min<size_t>(batch, n - b0);
         CUDA_TRY(launch_rows_gather(rows, M->Fpad, M->idx_all + b0, M->Xd, M->Xb, M->O, M->Td, M->Tb, M->s));
-        M->forward(M->Xb, rows, M->Y, M->H1, M->H2, M->s);
-        M->backward(M->Xb, M->Tb, rows);
+        M->train_pass(nullptr, M->Tb, rows);
         M->adam_t += 1;
         CUDA_TRY(launch_adam((int)M->nparam, M->P, M->G, M->Am, M->Av, M->weights(), lr, 0.9f, 0.999f, 1e-8f, M->adam_t, M->s));
         CUDA_TRY(launch_colsum(152, 1, M->loss_part, M->loss_tmp, M->s));

@@ -396,7 +396,16 @@ struct MlpTile {
   const __nv_bfloat16 *Xb, *W1, *W2, *W3;
   const float *b1, *b2, *b3;
   float* Y;
+  // training pass (T non-null): the targets, 1 / (rows O); BF16 copies for the weight gradients: Xs
+  // [rows][Fpad] (from Xf), H1, H2, dZ2, dZ1 [rows][Hp], dY [rows][Op]; per-CTA column sums of dZ1, dZ2, dY
+  // [ctas][2 Hp + Op] and squared errors [kLossParts]
+  const float* T;
+  float inv_count;
+  __nv_bfloat16 *Xs, *H1, *H2, *dY, *dZ2, *dZ1;
+  float *bias_part, *loss_part;
 };
+constexpr int kLossParts = 152;    // one per SM
+int mlp_fused_ctas(int rows);
 bool mlp_fused_fits(int Hp, int Op);
 cudaError_t launch_mlp_fused(const MlpTile& P, cudaStream_t s);
 // The BF16 copies of the weight matrices W1 [Fpad][Hp], W2 [Hp][Hp], W3 [Hp][Op] (inputs x outputs,
@@ -407,6 +416,23 @@ struct MlpWeights {
   __nv_bfloat16 *W[3], *T[3];
   int H, O, Hp, Op, ob1, oW2, ob2, oW3, ob3;
 };
+// The weight-gradient products g = A^T B over the batch rows (A [rows][lda], M columns used; B [rows][ldb],
+// N columns; 16-byte aligned, lda and ldb multiples of 8) as partial sums over `splits` ranges of
+// split_rows rows (a multiple of 64): part[k * part_stride + out + m * N + n].
+struct WgradArgs {
+  struct Gemm {
+    const __nv_bfloat16 *A, *B;
+    int lda, M, ldb, N, tiles_m, tiles_n;
+    size_t out;
+  } g[3];
+  int rows, splits, split_rows;
+  size_t part_stride;
+  float* part;
+};
+// The products, then G[0, n): the weights' sums over the splits and the biases' over the CTAs of the
+// training pass.
+cudaError_t launch_wgrad(const WgradArgs& P, int n, int ctas, const float* bias_part, const MlpWeights& M, float* G,
+                         cudaStream_t s);
 cudaError_t launch_mse_grad(int rows, int O, const float* Y, const float* T, float* dYf, __nv_bfloat16* dYb,
                             float inv_count, float* loss_partial, int nblk, cudaStream_t s);
 cudaError_t launch_relu_mask(int n, float* dH, const __nv_bfloat16* H, __nv_bfloat16* dZb, cudaStream_t s);

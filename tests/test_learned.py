@@ -256,3 +256,22 @@ def test_forward_edges_match_mma_sync(dim, p, hidden, rows):
     gm.gemm_backend(1)
     ref = gm.forward(X)
     assert torch.isfinite(y).all() and (y - ref).norm() <= 2.0 ** -8 * ref.norm()
+
+
+@pytest.mark.parametrize("dim,p,hidden,rows", [(2, 1, 8, 1), (2, 2, 33, 127), (3, 1, 200, 129), (3, 2, 256, 300),
+                                               (2, 1, 264, 140), (2, 3, 128, 1111), (2, 1, 32, 152 * 128 + 5)])
+def test_training_pass_edges_match_mma_sync(dim, p, hidden, rows):
+    """The one-launch training pass with split weight gradients against the mma.sync layers, as above; the
+    gradients round twice (activations, backward products), each at most one BF16 unit of one value."""
+    import paper_2506_12899_gb300 as S
+    gm = S.Mlp(dim, p, hidden, seed=5)
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    X = torch.rand((rows, gm.F), generator=g, device="cuda") * 2 - 1
+    T = torch.randn((rows, gm.O), generator=g, device="cuda")
+    loss, grad = gm.gradients(X, T)
+    again, grad2 = gm.gradients(X, T)
+    assert loss == again and np.array_equal(grad, grad2)              # fixed-order sums
+    gm.gemm_backend(1)
+    ref_loss, ref = gm.gradients(X, T)
+    assert abs(loss - ref_loss) <= 2.0 ** -8 * ref_loss
+    assert np.linalg.norm(grad - ref) <= 2.0 ** -7 * np.linalg.norm(ref)
