@@ -1685,9 +1685,12 @@ int sbm_gram_schmidt(void* ctx, int variant, const double* V_dev, int nv, const 
     const double* one = C->gsdots + 65;
     double* col = C->gsdots + 128;
     // w into the padded buffer (the staged copies read whole 16-byte units past an odd N)
-    CUDA_TRY(cudaMemsetAsync(C->gsw, 0, ldv * sizeof(double), s));
-    CUDA_TRY(cudaMemcpyAsync(C->gsw, w_dev, N * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    auto copy_w = [&] {
+      CUDA_TRY(cudaMemsetAsync(C->gsw, 0, ldv * sizeof(double), s));
+      CUDA_TRY(cudaMemcpyAsync(C->gsw, w_dev, N * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    };
     if (variant == 2) {                              // FP64 basis: the sweeps of krylov_basis = 1
+      copy_w();
       CUDA_TRY(launch_multi_dot(V_dev, N, nv, C->gsw, N, C->gspartial, h1, 0, s));
       CUDA_TRY(launch_axpy_dot(V_dev, N, nv, h1, C->gsw, N, C->gspartial, h2, s));
       CUDA_TRY(launch_axpy_norm(V_dev, N, nv, h2, C->gsw, N, C->gspartial, hn, s));
@@ -1700,6 +1703,9 @@ int sbm_gram_schmidt(void* ctx, int variant, const double* V_dev, int nv, const 
       for (int k = 0; k < nv; ++k)                   // rows rounded to double-float (exact split)
         CUDA_TRY((launch_gs_scale<double, double>(V_dev + (size_t)k * N, one, C->gsV2 + (size_t)k * ldv,
                                                   (double*)nullptr, N, s)));
+      // The sweeps read V before their dependency wait, so its last row must not come from the launch
+      // just before them: the copies of w in between (no programmatic launch crosses a copy) see to that.
+      copy_w();
       if (variant == 1) {                            // w handed over as double-float (FP32-V-cycle solves)
         CUDA_TRY(cudaMemsetAsync(C->gswdf, 0, ldv * sizeof(float2), s));
         CUDA_TRY((launch_gs_scale<double, double>(C->gsw, one, C->gswdf, (double*)nullptr, N, s)));
