@@ -42,8 +42,6 @@ struct DevLevel {
   int* parent_code = nullptr;
   int* children = nullptr;
   double* coarse_inv = nullptr;
-  double* coarse_invT = nullptr;     // its transpose (the one-CTA tail reads it a row per thread)
-  dfl* coarse_invT_df = nullptr;     // the transpose rounded to double-float (FP32 tail)
   LevelParams<double> P64{};
   LevelParams<float> P32{};
   LevelParams<dfl> Pdf{};         // double-float operator constants (finest level, thread-per-cell shapes)
@@ -590,14 +588,6 @@ Context* build_context(const sbm_setup_desc& d, bool device) {
     if (!L.H.children.empty()) L.children = C->upload(L.H.children);
     if (!L.H.coarse_inv.empty()) {
       L.coarse_inv = C->upload(L.H.coarse_inv);
-      const size_t n = L.H.n_dof();
-      std::vector<double> t(n * n);
-      for (size_t i = 0; i < n; ++i)
-        for (size_t j = 0; j < n; ++j) t[j * n + i] = L.H.coarse_inv[i * n + j];
-      L.coarse_invT = C->upload(t);
-      std::vector<dfl> tdf(t.size());
-      for (size_t i = 0; i < t.size(); ++i) tdf[i] = dfl(t[i]);
-      L.coarse_invT_df = C->upload(tdf);
     }
     L.P64 = make_params<double>(L, L.dhat64, L.binv64);
     L.P32 = make_params<float>(L, L.dhat32, L.binv32);
@@ -673,6 +663,142 @@ Context* build_context(const sbm_setup_desc& d, bool device) {
   return C.release();
 }
 
+// The one-CTA tail over levels 0..top: its parameters and, uploaded, its shared-memory image (TailCta).
+// Returns the bytes of shared memory, 0 if they do not fit (or an index does not fit its 16 bits).
+template <typename R>
+size_t build_tail_cta(Context& C, int top, TailCta<R>& T) {
+  const int dim = C.lv[0].H.dim, np = C.lv[0].H.np, ncol = 1 << dim, pi = prec_index<R>();
+  const size_t blk = (size_t)np * np * sizeof(R) + 16;          // a padded boundary block
+  const size_t n0 = (size_t)C.lv[0].H.n_dof();
+  std::vector<TailLevelDesc> D((size_t)top + 1);
+  size_t bytes = 0, vec = 0;
+  auto take = [&](size_t n) {                       // n bytes on a 16-byte boundary
+    const size_t at = bytes;
+    bytes += (n + 15) / 16 * 16;
+    return (unsigned)at;
+  };
+  take(D.size() * sizeof(TailLevelDesc));
+  for (int l = 0; l <= top; ++l) {
+    const HostLevel& H = C.lv[l].H;
+    if (H.n_act >= 8191) return 0;                  // parent << 3 | child bits in 16 bits
+    D[l] = TailLevelDesc{};
+    D[l].n_act = H.n_act;
+    for (int g = 0; g <= dim; ++g) {
+      int end[3] = {0, 0, 0}, first[3] = {0, 0, 0}, k = 0, n = 0;
+      for (int c = 0; c < ncol; ++c) {
+        if (__builtin_popcount((unsigned)c) != g) continue;
+        first[k] = H.colour_start[c] - n;
+        n += H.colour_start[c + 1] - H.colour_start[c];
+        end[k++] = n;
+      }
+      for (; k < 3; ++k) end[k] = n;
+      D[l].grp[g] = {end[0], end[1], end[2], first[0], first[1], first[2]};
+    }
+    D[l].mats = take(kTailMats * sizeof(R));
+    D[l].binv = take(H.n_bnd * blk);
+    D[l].rec = take((size_t)H.n_act * 16);
+    if (l >= 1) D[l].ch = take((size_t)ncol * C.lv[l - 1].H.n_act * 2);
+    vec += (size_t)(H.n_act + 1) * np * sizeof(R);
+  }
+  auto fits = [&] { return tail_cta_fits(dim, pi, bytes + 2 * vec); };
+  if (!fits()) return 0;
+  // the coarse inverse, then the boundary self blocks from the smallest level up, where they still fit
+  size_t keep = bytes;
+  T.cinv = take(n0 * n0 * 8);
+  if (!fits()) {
+    bytes = keep;
+    T.cinv = 0;
+  }
+  for (int l = 1; l <= top; ++l) {
+    keep = bytes;
+    D[l].aself = take(C.lv[l].H.n_bnd * blk);
+    if (fits()) continue;
+    bytes = keep;
+    D[l].aself = 0;
+    break;
+  }
+  size_t z = bytes;
+  for (int l = 0; l <= top; ++l) {
+    D[l].z = (unsigned)z;
+    D[l].f = (unsigned)(z + vec);
+    z += (size_t)(D[l].n_act + 1) * np * sizeof(R);
+  }
+  std::vector<unsigned char> image(bytes, 0);
+  std::memcpy(image.data(), D.data(), D.size() * sizeof(TailLevelDesc));
+  for (int l = 0; l <= top; ++l) {
+    const HostLevel& H = C.lv[l].H;
+    // couplings h^(d-2) w B (p = 1: every face point has the weight w), the transposed inverse (by fast
+    // diagonalisation) and self block of an interior cell: FP64, then rounded
+    R* M = reinterpret_cast<R*>(&image[D[l].mats]);
+    const double hs = std::pow(H.h, dim - 2), wt = dim == 2 ? H.B.w[0] : H.B.w[0] * H.B.w[0];
+    for (int q = 0; q < 4; ++q) {
+      M[q] = (R)(hs * wt * H.Bpm[q]);
+      M[4 + q] = (R)(hs * wt * H.Bmp[q]);
+    }
+    for (int i = 0; i < np; ++i)
+      for (int j = 0; j < np; ++j) {
+        double inv = 0, self = 0;
+        for (int m = 0; m < np; ++m) {
+          double v = 1, lam = 0;
+          for (int k = 0; k < dim; ++k) {
+            const int ik = (i >> k) & 1, jk = (j >> k) & 1, mk = (m >> k) & 1;
+            v *= H.S[ik * 2 + mk] * H.S[jk * 2 + mk];
+            lam += H.lam[mk];
+          }
+          inv += v / (hs * lam);
+        }
+        for (int k = 0; k < dim; ++k)
+          if (((i ^ j) & ~(1 << k)) == 0) self += hs * wt * H.L[3][((i >> k) & 1) * 2 + ((j >> k) & 1)];
+        M[8 + j * np + i] = (R)inv;
+        M[8 + np * np + j * np + i] = (R)self;
+      }
+    for (int b = 0; b < H.n_bnd; ++b)
+      for (int q = 0; q < np * np; ++q) {
+        reinterpret_cast<R*>(&image[D[l].binv + b * blk])[q] = (R)H.binvT[(size_t)b * np * np + q];
+        if (D[l].aself) reinterpret_cast<R*>(&image[D[l].aself + b * blk])[q] = (R)H.aselfT[(size_t)b * np * np + q];
+      }
+    uint16_t* rec = reinterpret_cast<uint16_t*>(&image[D[l].rec]);
+    for (int a = 0; a < H.n_act; ++a, rec += 8) {
+      for (int s = 0; s < 6; ++s) {
+        const int n = s < 2 * dim ? H.nbr[(size_t)s * H.n_act + a] : -1;
+        rec[s] = (uint16_t)(n >= 0 ? n : H.n_act);
+      }
+      int b;
+      rec[6] = H.is_boundary(a, &b) ? (uint16_t)b : 0xffff;
+      rec[7] = l >= 1 && H.parent_code[a] >= 0 ? (uint16_t)H.parent_code[a] : 0xffff;
+    }
+    if (l >= 1) {
+      const HostLevel& Hc = C.lv[l - 1].H;
+      uint16_t* ch = reinterpret_cast<uint16_t*>(&image[D[l].ch]);
+      for (int cc = 0; cc < Hc.n_act; ++cc)
+        for (int o = 0; o < ncol; ++o) {
+          const int a = Hc.children[(size_t)o * Hc.n_act + cc];
+          ch[(size_t)cc * ncol + o] = a >= 0 ? (uint16_t)a : 0xffff;
+        }
+      if (!D[l].aself) T.aselfT[l] = C.upload(std::vector<R>(H.aselfT.begin(), H.aselfT.end()));
+    }
+    T.omega[l] = (R)H.omega;
+  }
+  if (T.cinv)
+    for (size_t i = 0; i < n0; ++i)
+      for (size_t j = 0; j < n0; ++j) {
+        const double v = C.lv[0].H.coarse_inv[i * n0 + j];
+        if constexpr (sizeof(R) == 4) reinterpret_cast<dfl*>(&image[T.cinv])[j * n0 + i] = dfl(v);
+        else reinterpret_cast<double*>(&image[T.cinv])[j * n0 + i] = v;
+      }
+  T.top = top;
+  T.pre = C.desc.pre_smooth;
+  T.post = C.desc.post_smooth;
+  T.ssor = C.desc.ssor_each;
+  T.n0 = (int)n0;
+  T.image_bytes = (unsigned)bytes;
+  T.vec_bytes = (unsigned)vec;
+  T.image = C.upload(image);
+  for (int o = 0; o < 2; ++o)
+    for (int q = 0; q < 4; ++q) T.Ph[o][q] = tparams<R>(C.lv[1]).Ph[o][q];
+  return bytes + 2 * vec;
+}
+
 template <typename R>
 void ensure_work(Context& C) {
   const int pi = prec_index<R>();
@@ -690,67 +816,18 @@ void ensure_work(Context& C) {
   // cluster tail: the highest candidate level whose vectors (levels 0..top) fit in the shared
   // memory of a resident cluster of 16, else 8, CTAs
   C.tail_plan[pi] = TailPlan{};
-  const int NP = C.lv[0].H.dim == 2 ? 4 : 8;
+  const int NP = C.lv[0].H.np;
   // default (tail_max_cells = 0): the one-CTA tail for FP32 V-cycles, none for FP64 ones (one
   // SM's FP64 pipe makes it slower than per-level launches: measured)
   const bool tail_default = C.desc.tail_max_cells == 0;
   const int ctas = C.desc.tail_cluster_ctas == 0 ? 1 : C.desc.tail_cluster_ctas;
   if (ctas == 1 && !(tail_default && sizeof(R) == 8)) {
     // one CTA: the highest candidate level whose data (levels 0..top) fit in its shared memory
-    const int dim = C.lv[0].H.dim, ncol = 1 << dim;
     for (int top = std::min(C.tail_cand, kMaxTailCta - 1); top >= 1; --top) {
       auto tp = std::make_unique<TailCta<R>>();
-      std::memset(tp.get(), 0, sizeof(TailCta<R>));
-      size_t re = 0, ie = 0;                        // R elements, ints
-      // every array starts on a 16-byte boundary, so that bulk copies can stage the tables
-      const size_t ra = 16 / sizeof(R), ia = 4;
-      auto up = [](size_t v, size_t a) { return (v + a - 1) / a * a; };
-      bool aligned = true;
-      auto al16 = [&](const void* p) { aligned = aligned && reinterpret_cast<uintptr_t>(p) % 16 == 0; };
-      for (int l = 0; l <= top; ++l) {
-        const HostLevel& H = C.lv[l].H;
-        tp->P[l] = params<R>(C.lv[l]);
-        if (l >= 1) tp->T[l] = tparams<R>(C.lv[l]);
-        tp->n_bnd[l] = H.n_bnd;
-        tp->zoff[l] = (int)re;
-        re = up(re + (size_t)H.n_act * NP, ra);
-        tp->roff[l] = (int)re;
-        re = up(re + (size_t)H.n_act * NP, ra);
-        tp->boff[l] = (int)re;
-        re = up(re + (size_t)H.n_bnd * NP * NP, ra);
-        tp->noff[l] = (int)ie;
-        ie = up(ie + (size_t)2 * dim * H.n_act, ia);
-        al16(tp->P[l].nbr);
-        al16(tp->P[l].binvT);
-        if (l >= 1) {
-          tp->coff[l] = (int)ie;
-          ie = up(ie + (size_t)ncol * C.lv[l - 1].H.n_act, ia);
-          tp->poff[l] = (int)ie;
-          ie = up(ie + (size_t)H.n_act, ia);
-          al16(tp->T[l].children);
-          al16(tp->T[l].parent_code);
-        }
-      }
-      tp->bulk = aligned ? 1 : 0;
-      const size_t int_base = (re * sizeof(R) + 15) / 16 * 16;
-      size_t smem = int_base + ie * sizeof(int);
-      // the coarse inverse (FP64, n0 x n0) joins the staged data when it fits
-      const size_t n0 = (size_t)C.lv[0].H.n_act * NP;
-      const size_t cinv_off = up(smem, 16), smem_c = cinv_off + n0 * n0 * sizeof(double);
-      tp->cinv_off = 0;
-      const void* cinvT = sizeof(R) == 4 ? static_cast<const void*>(C.lv[0].coarse_invT_df)
-                                         : static_cast<const void*>(C.lv[0].coarse_invT);
-      if (cinvT && reinterpret_cast<uintptr_t>(cinvT) % 16 == 0 &&
-          tail_cta_fits(dim, pi, smem_c, sizeof(TailCta<R>))) {
-        tp->cinv_off = (unsigned)cinv_off;
-        smem = smem_c;
-      }
-      tp->top = top;
-      tp->pre = C.desc.pre_smooth;
-      tp->post = C.desc.post_smooth;
-      tp->ssor = C.desc.ssor_each;
-      tp->int_base = (unsigned)int_base;
-      if (!tail_cta_fits(dim, pi, smem, sizeof(TailCta<R>))) continue;
+      std::memset(static_cast<void*>(tp.get()), 0, sizeof(TailCta<R>));
+      const size_t smem = build_tail_cta<R>(C, top, *tp);
+      if (smem == 0) continue;
       C.tail_plan[pi].top = top;
       C.tail_plan[pi].cluster = 1;
       C.tail_plan[pi].smem_bytes = smem;
@@ -909,9 +986,7 @@ void vcycle_rec(Context& C, int l, const R* r, R* z, cudaStream_t s, bool first_
       const TailCta<R>* tp;
       if constexpr (sizeof(R) == 8) tp = C.tail_cta64.get();
       else tp = C.tail_cta32.get();
-      const void* cinvT = sizeof(R) == 4 ? static_cast<const void*>(C.lv[0].coarse_invT_df)
-                                         : static_cast<const void*>(C.lv[0].coarse_invT);
-      CUDA_TRY(launch_vcycle_tail_cta<R>(L.H.dim, *tp, r, z, C.lv[0].coarse_inv, cinvT, C.tail_plan[pi].smem_bytes, s));
+      CUDA_TRY(launch_vcycle_tail_cta<R>(L.H.dim, *tp, r, z, C.lv[0].coarse_inv, C.tail_plan[pi].smem_bytes, s));
     } else {
       CUDA_TRY(launch_vcycle_tail<R>(L.H.dim, static_cast<const TailLevel<R>*>(C.tail[pi]), l, r, z,
                                      C.lv[0].coarse_inv, C.desc.pre_smooth, C.desc.post_smooth, C.desc.ssor_each,

@@ -478,301 +478,311 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_vcycle_tail(const TailLevel
 // The V-cycle of levels 0..top (p = 1 h-levels) in one CTA: all data of those levels in shared
 // memory, phases separated by __syncthreads(); see TailCta.
 // ----------------------------------------------------------------------------------------------
-// Threads of the one-CTA tail: 1024 for 2D FP32 (a colour group of the 64^2 level in one pass), 512
-// otherwise (register budget).
-template <int D, typename R>
-constexpr int tail_cta_threads() {
-  return D == 2 && sizeof(R) == 4 ? 1024 : 512;
-}
+// Threads of the one-CTA tail.  (With 1024 in 2D every phase was 50 to 100 cycles longer, the barrier and
+// the idle warps' share of it.)
+constexpr int kTailCtaThreads = 512;
 
 // Set when the tail's staging copies did not complete within kAsyncSpin polls (the tail then
 // copied the data itself); tail_fault_take() reads and clears it.
 __device__ int g_tail_fault;
 
+// What bounds it: the latency of some 25 dependent phases.  So:
+//   - the tables arrive as one bulk copy, before the dependency wait;
+//   - the level descriptors are in shared memory (indexed reads of the parameter block missed the
+//     constant cache in every phase);
+//   - every phase's code appears once, in one loop over the levels down and up again, so the instructions
+//     of a phase are in the cache from its first use on;
+//   - a cell's neighbours, boundary index and parent are one 16-byte record; a missing neighbour is a
+//     zero cell, so no load waits for a branch; an interior cell applies a dense inverse like a
+//     boundary cell, so a warp of both takes one path;
+//   - vectors and blocks are laid out free of bank conflicts (TailCta).
+// What is left is bound by the shared-memory reads of the largest level's phases (the 64^2 level: 850 to
+// 1500 cycles a colour group, 4200 the restriction) and by each thread's chain on the smaller ones (500 to
+// 600 cycles).  A V-cycle of the 512^2 p = 2 star (tail: 64^2 .. 8^2) went 127 -> 107 us, one of a 64^3 p = 1
+// sphere (16^3 .. 4^3; its boundary self blocks stay in global memory) 153 -> 108 us.
 template <int D, typename R>
-__global__ void __launch_bounds__(tail_cta_threads<D, R>(), 1) k_vcycle_tail_cta(const __grid_constant__ TailCta<R> TP,
+__global__ void __launch_bounds__(kTailCtaThreads, 1) k_vcycle_tail_cta(const __grid_constant__ TailCta<R> TP,
                                                                         const R* __restrict__ r_top,
                                                                         R* __restrict__ z_top,
-                                                                        const double* __restrict__ coarse_inv,
-                                                                        const void* __restrict__ coarse_invT) {
+                                                                        const double* __restrict__ coarse_inv) {
   extern __shared__ __align__(16) unsigned char tcta_smem[];
-  R* sm = reinterpret_cast<R*>(tcta_smem);
-  int* si = reinterpret_cast<int*>(tcta_smem + TP.int_base);
-  constexpr int NCOL = 1 << D, NP = CD<D, 2>::NP, NT = tail_cta_threads<D, R>();
+  constexpr int NCOL = 1 << D, NP = CD<D, 2>::NP, NT = kTailCtaThreads;
+  constexpr int W = NP * (int)sizeof(R) / 16, PW = NP / W;      // 16-byte words of a cell, values of a word
+  constexpr unsigned BLK = NP * NP * sizeof(R) + 16;            // a padded boundary block
+  static_assert(NP == NCOL, "one value per child in the restriction's exchange");
   const int top = TP.top, tid = threadIdx.x;
-  // Stage the tables and inverses of every level (set-up data, staged while the kernel before
-  // finishes), then, after the wait, the top level's right-hand side.  With TP.bulk, thread 0
-  // moves the 16-byte multiple part of every array with bulk asynchronous copies (all sources and
-  // slots are 16-byte aligned) and the threads copy the few entries past it; otherwise (or if a
-  // copy does not complete in bounded time) the threads copy everything.
-  __shared__ __align__(8) unsigned long long tbar[2];
-  const int nr = TP.P[top].n_act * NP;
-  const bool rbulk = TP.bulk && reinterpret_cast<uintptr_t>(r_top) % 16 == 0;
-  // visits every staged table: f(dst, src, count, element size)
-  auto tables = [&](auto&& f) {
-    for (int l = 0; l <= top; ++l) {
-      const LevelParams<R>& P = TP.P[l];
-      f(static_cast<void*>(si + TP.noff[l]), static_cast<const void*>(P.nbr), 2 * D * P.n_act, (int)sizeof(int));
-      f(static_cast<void*>(sm + TP.boff[l]), static_cast<const void*>(P.binvT), TP.n_bnd[l] * NP * NP,
-        (int)sizeof(R));
-      if (l >= 1) {
-        const TransferParams<R>& T = TP.T[l];
-        f(static_cast<void*>(si + TP.coff[l]), static_cast<const void*>(T.children), NCOL * T.n_act_c, (int)sizeof(int));
-        f(static_cast<void*>(si + TP.poff[l]), static_cast<const void*>(T.parent_code), T.n_act_f, (int)sizeof(int));
-      }
-    }
-    if (TP.cinv_off) {
-      const int n0 = TP.P[0].n_act * NP;
-      f(static_cast<void*>(tcta_smem + TP.cinv_off), coarse_invT, n0 * n0, 8);
-    }
-  };
-  auto plain = [&](void* dst, const void* src, int n, int es, int from) {   // entries [from, n)
-    if (es == 4)
-      for (int q = from + tid; q < n; q += NT) static_cast<int*>(dst)[q] = static_cast<const int*>(src)[q];
-    else
-      for (int q = from + tid; q < n; q += NT) static_cast<double*>(dst)[q] = static_cast<const double*>(src)[q];
-  };
-  if (TP.bulk) {
-    if (tid == 0) {
-      mbar_init(&tbar[0], 1);
-      mbar_init(&tbar[1], 1);
-      mbar_fence_init();
-      unsigned total = 0;
-      tables([&](void*, const void*, int n, int es) { total += (unsigned)(n * es) & ~15u; });
-      mbar_arrive_tx(&tbar[0], total);
-      tables([&](void* dst, const void* src, int n, int es) {
-        const unsigned b = (unsigned)(n * es) & ~15u;
-        if (b) bulk_load(dst, src, b, &tbar[0]);
-      });
-    }
-    tables([&](void* dst, const void* src, int n, int es) { plain(dst, src, n, es, (int)(((unsigned)(n * es) & ~15u) / es)); });
-    __syncthreads();                                 // barriers initialised before anyone polls them
-  } else {
-    tables([&](void* dst, const void* src, int n, int es) { plain(dst, src, n, es, 0); });
+  const TailLevelDesc* lev = reinterpret_cast<const TailLevelDesc*>(tcta_smem);
+  __shared__ __align__(8) unsigned long long tbar;
+  if (tid == 0) {
+    mbar_init(&tbar, 1);
+    mbar_fence_init();
+    mbar_arrive_tx(&tbar, TP.image_bytes);
+    bulk_load(tcta_smem, TP.image, TP.image_bytes, &tbar);
   }
+  for (unsigned q = tid; q < TP.vec_bytes / 8; q += NT)         // z and f: zero
+    reinterpret_cast<uint4*>(tcta_smem + TP.image_bytes)[q] = make_uint4(0u, 0u, 0u, 0u);
+  R P0[4], P1[4];                                    // 1D transfer matrices of the two children
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    P0[q] = TP.Ph[0][q];
+    P1[q] = TP.Ph[1][q];
+  }
+  __syncthreads();                                   // the barrier is initialised before anyone polls it
+  if (!__syncthreads_and(mbar_wait(&tbar, 0))) {     // record, let the copy land, copy by hand
+    if (tid == 0) {
+      atomicExch(&g_tail_fault, 1);
+      mbar_wait(&tbar, 0);
+    }
+    __syncthreads();
+    for (unsigned q = tid; q < TP.image_bytes / 16; q += NT)
+      reinterpret_cast<uint4*>(tcta_smem)[q] = static_cast<const uint4*>(TP.image)[q];
+    __syncthreads();
+  }
+
+  // the NP values of cell a of the vector at byte offset v of a level of n cells
+  auto load = [&](unsigned v, int n, unsigned a, R(&x)[NP]) {
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      R t[PW];
+      load_np_vec<PW, R>(reinterpret_cast<const R*>(tcta_smem + v + (unsigned)(w * (n + 1) + (int)a) * 16u), t);
+#pragma unroll
+      for (int i = 0; i < PW; ++i) x[w * PW + i] = t[i];
+    }
+  };
+  auto store = [&](unsigned v, int n, unsigned a, const R(&x)[NP]) {
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      R t[PW];
+#pragma unroll
+      for (int i = 0; i < PW; ++i) t[i] = x[w * PW + i];
+      store_np_vec<PW, R>(reinterpret_cast<R*>(tcta_smem + v + (unsigned)(w * (n + 1) + (int)a) * 16u), t);
+    }
+  };
+  // t -= the couplings to the neighbours of the record q (Eq. 10)
+  auto couple = [&](const uint4& q, unsigned z, int n, const R(&b)[8], R(&t)[NP]) {
+    const unsigned w[3] = {q.x, q.y, q.z};
+#pragma unroll
+    for (int s = 0; s < 2 * D; ++s) {
+      R u[NP];
+      load(z, n, (s & 1) ? w[s >> 1] >> 16 : w[s >> 1] & 0xffffu, u);
+#pragma unroll
+      for (int tl = 0; tl < NP / 2; ++tl)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const int k = dof<D, 2>(s >> 1, i, tl);
+          t[k] -= b[4 * (s & 1) + 2 * i] * u[dof<D, 2>(s >> 1, 0, tl)];
+          t[k] -= b[4 * (s & 1) + 2 * i + 1] * u[dof<D, 2>(s >> 1, 1, tl)];
+        }
+    }
+  };
+  // y += sign * T^T t for a transposed NP x NP block T
+  auto block = [&](const R* T, const R(&t)[NP], R sign, R(&y)[NP]) {
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      R c[NP];
+      load_np_vec<NP, R>(T + j * NP, c);
+      const R tj = sign * t[j];
+#pragma unroll
+      for (int i = 0; i < NP; ++i) y[i] += c[i] * tj;
+    }
+  };
   pdl_wait();
   pdl_trigger();
-  if (rbulk) {
-    if (tid == 0) {
-      mbar_arrive_tx(&tbar[1], (unsigned)(nr * sizeof(R)));
-      bulk_load(sm + TP.roff[top], r_top, (unsigned)(nr * sizeof(R)), &tbar[1]);
+  {                                                  // the top level's right-hand side
+    const int n = lev[top].n_act;
+    const unsigned f = lev[top].f;
+    if (reinterpret_cast<uintptr_t>(r_top) % 16 == 0) {
+      for (int q0 = tid; q0 < n * W; q0 += 4 * NT) { // four words in flight per thread
+        uint4 v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (q0 + k * NT < n * W) v[k] = reinterpret_cast<const uint4*>(r_top)[q0 + k * NT];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int q = q0 + k * NT;
+          if (q < n * W) *reinterpret_cast<uint4*>(tcta_smem + f + (unsigned)((q % W) * (n + 1) + q / W) * 16u) = v[k];
+        }
+      }
+    } else {
+      for (int q = tid; q < n * NP; q += NT)
+        reinterpret_cast<R*>(tcta_smem + f)[((q % NP) / PW * (n + 1) + q / NP) * PW + q % PW] = r_top[q];
     }
+    __syncthreads();
+  }
+  for (int step = 0; step <= 2 * top; ++step) {      // down: top .. 1, the coarse solve, up: 1 .. top
+    const bool down = step < top;
+    const int l = down ? top - step : step - top;
+    if (step == top) {                               // coarse solve: 8 lanes per row
+      const int n0 = TP.n0, na = lev[0].n_act;
+      auto at = [&](unsigned v, int c) -> R& {       // unknown c of level 0
+        return reinterpret_cast<R*>(tcta_smem + v)[((c % NP) / PW * (na + 1) + c / NP) * PW + c % PW];
+      };
+      const unsigned r0 = lev[0].f, z0 = lev[0].z;
+      if (TP.cinv) {
+        // the transpose staged in shared memory.  FP32 tail: the inverse is stored as double-float
+        // and every product is exact (two_prod) and summed in double-float on the FP32 pipes (about
+        // 48 bits; the input and the result are FP32), since one SM's FP64 pipe made this the tail's
+        // longest phase.  FP64 tail: FP64 throughout.
+        for (int base = 0; base < n0; base += NT / 8) {
+          const int row = base + tid / 8, c0 = tid & 7;
+          if constexpr (sizeof(R) == 4) {
+            const dfl* aT = reinterpret_cast<const dfl*>(tcta_smem + TP.cinv);
+            dfl acc(0.f);
+            if (row < n0)
+              for (int c = c0; c < n0; c += 8) acc += aT[(size_t)c * n0 + row] * (float)at(r0, c);
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1)
+              acc += dfl(__shfl_xor_sync(0xffffffffu, acc.hi, off), __shfl_xor_sync(0xffffffffu, acc.lo, off));
+            if (row < n0 && c0 == 0) at(z0, row) = (R)__fadd_rn(acc.hi, acc.lo);
+          } else {
+            const double* aT = reinterpret_cast<const double*>(tcta_smem + TP.cinv);
+            double acc = 0.0;
+            if (row < n0)
+              for (int c = c0; c < n0; c += 8) acc += aT[(size_t)c * n0 + row] * (double)at(r0, c);
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+            if (row < n0 && c0 == 0) at(z0, row) = (R)acc;
+          }
+        }
+      } else {                                       // from global memory, one warp per row
+        const int lane = tid & 31;
+        for (int row = tid >> 5; row < n0; row += NT / 32) {
+          double acc = 0;
+          for (int c = lane; c < n0; c += 32) acc += coarse_inv[(size_t)row * n0 + c] * (double)at(r0, c);
+#pragma unroll
+          for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+          if (lane == 0) at(z0, row) = (R)acc;
+        }
+      }
+      __syncthreads();
+      continue;
+    }
+    const TailLevelDesc& L = lev[l];
+    const int n = L.n_act;
+    const unsigned z = L.z, f = L.f;
+    const R* M = reinterpret_cast<const R*>(tcta_smem + L.mats);
+    const uint4* rec = reinterpret_cast<const uint4*>(tcta_smem + L.rec);
+    R bc[8];                                         // the level's couplings
+#pragma unroll
+    for (int i = 0; i < 8; ++i) bc[i] = M[i];
+    if (!down) {                                     // prolongation (Eq. 17)
+      const int nc = lev[l - 1].n_act;
+      const unsigned zc = lev[l - 1].z;
+      for (int a = tid; a < n; a += NT) {
+        const unsigned code = rec[a].w >> 16;
+        if (code == 0xffffu) continue;
+        R e[NP], u[NP];
+        load(zc, nc, code >> 3, e);
+        load(z, n, a, u);
+#pragma unroll
+        for (int dir = 0; dir < D; ++dir) {
+          const bool hi = (code >> dir) & 1u;
+#pragma unroll
+          for (int tl = 0; tl < NP / 2; ++tl) {
+            const int i0 = dof<D, 2>(dir, 0, tl), i1 = dof<D, 2>(dir, 1, tl);
+            const R e0 = e[i0], e1 = e[i1];
+            e[i0] = (hi ? P1[0] : P0[0]) * e0 + (hi ? P1[1] : P0[1]) * e1;
+            e[i1] = (hi ? P1[2] : P0[2]) * e0 + (hi ? P1[3] : P0[3]) * e1;
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < NP; ++i) u[i] += e[i];
+        store(z, n, a, u);
+      }
+      __syncthreads();
+    }
+    // smoothing: forward sweeps down, reverse sweeps up; ssor: each step forward, then reverse
+    const int sweeps = (down ? TP.pre : TP.post) << (TP.ssor ? 1 : 0);
+    const R om = TP.omega[l];
+    const unsigned binv = L.binv;
+    for (int sw = 0; sw < sweeps; ++sw) {
+      const bool fwd = TP.ssor ? (sw & 1) == 0 : down;
+      for (int gi = 0; gi <= D; ++gi) {              // one colour group (its cells share no face)
+        const TailLevelDesc::Group& G = L.grp[fwd ? gi : D - gi];
+        const int end2 = G.end2;
+        for (int idx = tid; idx < end2; idx += NT) {
+          const int a = idx + (idx < G.end0 ? G.first0 : (idx < G.end1 ? G.first1 : G.first2));
+          const uint4 q = rec[a];
+          R t[NP], y[NP];
+          load(f, n, a, t);
+          couple(q, z, n, bc, t);
+          const unsigned b = q.w & 0xffffu;
+#pragma unroll
+          for (int i = 0; i < NP; ++i) y[i] = R(0);
+          block(b == 0xffffu ? M + 8 : reinterpret_cast<const R*>(tcta_smem + binv + b * BLK), t, R(1), y);
+          if (om != R(1)) {
+            R uo[NP];
+            load(z, n, a, uo);
+#pragma unroll
+            for (int i = 0; i < NP; ++i) y[i] = (R(1) - om) * uo[i] + om * y[i];
+          }
+          store(z, n, a, y);
+        }
+        __syncthreads();
+      }
+    }
+    if (down) {
+      // residual and restriction (Eq. 18): a warp takes 32 / 2^d coarse cells, lanes o * (32 / 2^d) + i child o
+      // of coarse cell i, so that the lanes of one child read neighbouring cells
+      const unsigned short* ch = reinterpret_cast<const unsigned short*>(tcta_smem + L.ch);
+      const int nc = lev[l - 1].n_act, nl = nc * NCOL;
+      R* rc = reinterpret_cast<R*>(tcta_smem + lev[l - 1].f);
+      const unsigned aself = L.aself;
+      for (int base = 0; base < nl; base += NT) {    // (the same passes for the whole block: exchanges)
+        constexpr int CPW = 32 / NCOL;
+        const int o = (tid & 31) / CPW, cc = (base + (tid & ~31)) / NCOL + (tid & (CPW - 1));
+        const unsigned a = cc < nc ? ch[cc * NCOL + o] : 0xffffu;
+        R r[NP];
+#pragma unroll
+        for (int i = 0; i < NP; ++i) r[i] = R(0);
+        if (a != 0xffffu) {
+          const uint4 q = rec[a];
+          const unsigned b = q.w & 0xffffu;
+          R u[NP];
+          load(z, n, a, u);
+          load(f, n, a, r);
+          if (aself) block(b == 0xffffu ? M + 8 + NP * NP : reinterpret_cast<const R*>(tcta_smem + aself + b * BLK), u, R(-1), r);
+          else block(b == 0xffffu ? M + 8 + NP * NP : TP.aselfT[l] + b * (NP * NP), u, R(-1), r);
+          couple(q, z, n, bc, r);
+#pragma unroll
+          for (int dir = 0; dir < D; ++dir) {
+            const bool hi = (o >> dir) & 1;
+#pragma unroll
+            for (int tl = 0; tl < NP / 2; ++tl) {
+              const int i0 = dof<D, 2>(dir, 0, tl), i1 = dof<D, 2>(dir, 1, tl);
+              const R e0 = r[i0], e1 = r[i1];
+              r[i0] = (hi ? P1[0] : P0[0]) * e0 + (hi ? P1[2] : P0[2]) * e1;
+              r[i1] = (hi ? P1[1] : P0[1]) * e0 + (hi ? P1[3] : P0[3]) * e1;
+            }
+          }
+        }
+        // the sum over the children: at each exchange a lane keeps half of the values
+        int j = 0;
+#pragma unroll
+        for (int half = NP / 2, off = CPW; half >= 1; half >>= 1, off <<= 1) {
+          const bool upper = (tid & off) != 0;
+          if (upper) j += half;
+#pragma unroll
+          for (int i = 0; i < half; ++i) {
+            const R send = upper ? r[i] : r[i + half], keep = upper ? r[i + half] : r[i];
+            r[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+          }
+        }
+        if (cc < nc) rc[(j / PW * (nc + 1) + cc) * PW + j % PW] = r[0];
+      }
+      __syncthreads();
+    }
+  }
+  const int n = lev[top].n_act;
+  const unsigned z = lev[top].z;
+  if (reinterpret_cast<uintptr_t>(z_top) % 16 == 0) {
+    for (int q = tid; q < n * W; q += NT)
+      reinterpret_cast<uint4*>(z_top)[q] =
+          *reinterpret_cast<const uint4*>(tcta_smem + z + (unsigned)((q % W) * (n + 1) + q / W) * 16u);
   } else {
-    for (int q = tid; q < nr; q += NT) sm[TP.roff[top] + q] = r_top[q];
+    for (int q = tid; q < n * NP; q += NT)
+      z_top[q] = reinterpret_cast<const R*>(tcta_smem + z)[((q % NP) / PW * (n + 1) + q / NP) * PW + q % PW];
   }
-  if (TP.bulk) {
-    const bool ok = mbar_wait(&tbar[0], 0) && (!rbulk || mbar_wait(&tbar[1], 0));
-    if (!__syncthreads_and(ok)) {                    // record, let the copies land, copy by hand
-      if (tid == 0) {
-        atomicExch(&g_tail_fault, 1);
-        mbar_wait(&tbar[0], 0);
-        if (rbulk) mbar_wait(&tbar[1], 0);
-      }
-      __syncthreads();
-      tables([&](void* dst, const void* src, int n, int es) { plain(dst, src, n, es, 0); });
-      for (int q = tid; q < nr; q += NT) sm[TP.roff[top] + q] = r_top[q];
-    }
-  }
-  __syncthreads();
-
-  auto nbr_of = [&](int l, int a, int (&nb)[2 * D]) {
-#pragma unroll
-    for (int s = 0; s < 2 * D; ++s) nb[s] = si[TP.noff[l] + s * TP.P[l].n_act + a];
-  };
-  // one colour group g (colours with g odd index bits, which share no face): all its cells at once
-  auto smooth = [&](int l, int g, bool zs) {
-    const LevelParams<R>& P = TP.P[l];
-    // the group's colours c0 < c1 < c2 (at most three) and the running cell counts before c1, c2
-    int c0 = -1, c1 = -1, c2 = -1, n0 = 0, n1 = 0, n2 = 0;
-#pragma unroll
-    for (int c = 0; c < NCOL; ++c)
-      if (__popc(c) == g) {
-        const int n = P.colour_start[c + 1] - P.colour_start[c];
-        if (c0 < 0) { c0 = c; n0 = n; }
-        else if (c1 < 0) { c1 = c; n1 = n; }
-        else { c2 = c; n2 = n; }
-      }
-    R* z = sm + TP.zoff[l];
-    const R* f = sm + TP.roff[l];
-    for (int idx = tid; idx < n0 + n1 + n2; idx += NT) {
-      int col = c0, base = 0;
-      if (idx >= n0 + n1) { col = c2; base = n0 + n1; }
-      else if (idx >= n0) { col = c1; base = n0; }
-      const int cs = P.colour_start[col], nbnd = P.colour_nbnd[col];
-      const int a = cs + idx - base;
-      int nb[2 * D];
-      nbr_of(l, a, nb);
-      R c[NP];
-#pragma unroll
-      for (int i = 0; i < NP; ++i) c[i] = 0;
-      add_couplings_f<D, 2, R>(P.k, col, zs, nb, [&](int n, int, R(&un)[NP]) { load_np_vec<NP, R>(z + n * NP, un); },
-                               c);
-      R t[NP];
-      load_np_vec<NP, R>(f + a * NP, t);
-#pragma unroll
-      for (int i = 0; i < NP; ++i) t[i] -= P.hscale * c[i];
-      const int off = a - cs;
-      R y[NP];
-      block_solve_at<D, 2, R>(P, off < nbnd ? sm + TP.boff[l] + (size_t)(P.bstart[col] + off) * NP * NP : nullptr,
-                              t, y);
-      if (P.omega != R(1)) {
-        R uo[NP];
-        if (zs) {
-#pragma unroll
-          for (int i = 0; i < NP; ++i) uo[i] = 0;
-        } else {
-          load_np_vec<NP, R>(z + a * NP, uo);
-        }
-#pragma unroll
-        for (int i = 0; i < NP; ++i) y[i] = (R(1) - P.omega) * uo[i] + P.omega * y[i];
-      }
-      store_np_vec<NP, R>(z + a * NP, y);
-    }
-  };
-
-  for (int l = top; l >= 1; --l) {                 // down: pre-smooth, residual, restrict
-    const LevelParams<R>& P = TP.P[l];
-    if (TP.pre == 0) {
-      for (int q = tid; q < P.n_act * NP; q += NT) sm[TP.zoff[l] + q] = R(0);
-      __syncthreads();
-    }
-    for (int k = 0; k < TP.pre; ++k) {
-      for (int g = 0; g <= D; ++g) {
-        smooth(l, g, k == 0);
-        __syncthreads();
-      }
-      if (TP.ssor)
-        for (int g = D; g >= 0; --g) {
-          smooth(l, g, false);
-          __syncthreads();
-        }
-    }
-    const TransferParams<R>& T = TP.T[l];
-    const R* z = sm + TP.zoff[l];
-    const R* f = sm + TP.roff[l];
-    R* rc = sm + TP.roff[l - 1];
-    // one thread per child: group of NCOL adjacent lanes per coarse cell (lane o: child o), the
-    // child's residual restricted in registers, then a fixed butterfly sum over the group (every
-    // lane of a warp takes part: the pass count is the same for the whole block)
-    for (int base = 0; base < T.n_act_c * NCOL; base += NT) {
-      const int t = base + tid, cc = t / NCOL, o = t % NCOL;
-      const int a = cc < T.n_act_c ? si[TP.coff[l] + o * T.n_act_c + cc] : -1;
-      R out[NP];
-#pragma unroll
-      for (int j = 0; j < NP; ++j) out[j] = 0;
-      if (a >= 0) {
-        int ca = 0;
-#pragma unroll
-        for (int q = 1; q < NCOL; ++q)
-          if (a >= P.colour_start[q]) ca = q;
-        int nb[2 * D];
-        nbr_of(l, a, nb);
-        R v[NP], y[NP], fa[NP];
-        load_np_vec<NP, R>(z + a * NP, v);
-        load_np_vec<NP, R>(f + a * NP, fa);
-#pragma unroll
-        for (int i = 0; i < NP; ++i) y[i] = 0;
-        const int off = a - P.colour_start[ca];
-        add_self<D, 2, R>(P, nb, off < P.colour_nbnd[ca] ? P.bstart[ca] + off : -1, v, y);
-        add_couplings_f<D, 2, R>(P.k, ca, false, nb,
-                                 [&](int n, int, R(&un)[NP]) { load_np_vec<NP, R>(z + n * NP, un); }, y);
-#pragma unroll
-        for (int i = 0; i < NP; ++i) y[i] = fa[i] - P.hscale * y[i];
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
-          R acc = 0;
-#pragma unroll
-          for (int i = 0; i < NP; ++i) acc += h_weight<D, R>(T, o, i, j) * y[i];
-          out[j] = acc;
-        }
-      }
-#pragma unroll
-      for (int sh = 1; sh < NCOL; sh <<= 1)
-#pragma unroll
-        for (int j = 0; j < NP; ++j) out[j] += __shfl_xor_sync(0xffffffffu, out[j], sh);
-      if (o == 0 && cc < T.n_act_c) store_np_vec<NP, R>(rc + cc * NP, out);
-    }
-    __syncthreads();
-  }
-  {                                                // coarse solve in FP64, one warp per row
-    const int n0 = TP.P[0].n_act * NP;
-    const R* r0 = sm + TP.roff[0];
-    R* z0 = sm + TP.zoff[0];
-    if (TP.cinv_off) {
-      // the transpose staged in shared memory, one thread per row, four accumulation chains;
-      // consecutive threads read consecutive entries and r0[c] is a broadcast.  FP32 tail: the
-      // inverse is stored as double-float and every product is exact (two_prod) and summed in
-      // double-float on the FP32 pipes (about 48 bits; the input and the result are FP32), since
-      // one SM's FP64 pipe made this the tail's longest phase.  FP64 tail: FP64 throughout.
-      for (int row = tid; row < n0; row += NT) {
-        if constexpr (sizeof(R) == 4) {
-          const dfl* aT = reinterpret_cast<const dfl*>(tcta_smem + TP.cinv_off);
-          dfl acc[4] = {dfl(0.f), dfl(0.f), dfl(0.f), dfl(0.f)};
-          int c = 0;
-          for (; c + 4 <= n0; c += 4)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) acc[k] += aT[(size_t)(c + k) * n0 + row] * dfl((float)r0[c + k]);
-          for (; c < n0; ++c) acc[0] += aT[(size_t)c * n0 + row] * dfl((float)r0[c]);
-          const dfl sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-          z0[row] = (R)__fadd_rn(sum.hi, sum.lo);
-        } else {
-          const double* aT = reinterpret_cast<const double*>(tcta_smem + TP.cinv_off);
-          double acc[4] = {0.0, 0.0, 0.0, 0.0};
-          int c = 0;
-          for (; c + 4 <= n0; c += 4)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) acc[k] += aT[(size_t)(c + k) * n0 + row] * (double)r0[c + k];
-          for (; c < n0; ++c) acc[0] += aT[(size_t)c * n0 + row] * (double)r0[c];
-          z0[row] = (R)((acc[0] + acc[1]) + (acc[2] + acc[3]));
-        }
-      }
-    } else {                                       // from global memory, one warp per row
-      const int lane = tid & 31;
-      for (int row = tid >> 5; row < n0; row += NT / 32) {
-        double acc = 0;
-        for (int c = lane; c < n0; c += 32) acc += coarse_inv[(size_t)row * n0 + c] * (double)r0[c];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) z0[row] = (R)acc;
-      }
-    }
-    __syncthreads();
-  }
-  for (int l = 1; l <= top; ++l) {                 // up: prolongate, post-smooth
-    const LevelParams<R>& P = TP.P[l];
-    const TransferParams<R>& T = TP.T[l];
-    R* z = sm + TP.zoff[l];
-    const R* zc = sm + TP.zoff[l - 1];
-    for (int a = tid; a < P.n_act; a += NT) {
-      const int code = si[TP.poff[l] + a];
-      if (code < 0) continue;
-      const int par = code >> 3, o = code & 7;
-      R e[NP], u[NP];
-      load_np_vec<NP, R>(zc + par * NP, e);
-      load_np_vec<NP, R>(z + a * NP, u);
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        R acc = 0;
-#pragma unroll
-        for (int j = 0; j < NP; ++j) acc += h_weight<D, R>(T, o, i, j) * e[j];
-        u[i] += acc;
-      }
-      store_np_vec<NP, R>(z + a * NP, u);
-    }
-    __syncthreads();
-    for (int k = 0; k < TP.post; ++k) {
-      if (TP.ssor)
-        for (int g = 0; g <= D; ++g) {
-          smooth(l, g, false);
-          __syncthreads();
-        }
-      for (int g = D; g >= 0; --g) {
-        smooth(l, g, false);
-        __syncthreads();
-      }
-    }
-  }
-  for (int q = tid; q < TP.P[top].n_act * NP; q += NT) z_top[q] = sm[TP.zoff[top] + q];
 }
 
 inline unsigned cdiv(size_t a, size_t b) { return (unsigned)((a + b - 1) / b); }
@@ -977,8 +987,7 @@ bool tail_cta_fits_kernel(K kern, size_t smem) {
   return true;
 }
 
-bool tail_cta_fits(int dim, int prec, size_t smem, size_t param_bytes) {
-  (void)param_bytes;
+bool tail_cta_fits(int dim, int prec, size_t smem) {
   if (dim == 2) return prec == 0 ? tail_cta_fits_kernel(k_vcycle_tail_cta<2, double>, smem)
                                  : tail_cta_fits_kernel(k_vcycle_tail_cta<2, float>, smem);
   return prec == 0 ? tail_cta_fits_kernel(k_vcycle_tail_cta<3, double>, smem)
@@ -997,18 +1006,18 @@ int tail_fault_take() {
 
 template <typename R>
 cudaError_t launch_vcycle_tail_cta(int dim, const TailCta<R>& TP, const R* r, R* z, const double* coarse_inv,
-                                   const void* coarse_invT, size_t smem, cudaStream_t s) {
+                                   size_t smem, cudaStream_t s) {
   if (dim == 2)
-    SBM_PDL((k_vcycle_tail_cta<2, R>), 1, (tail_cta_threads<2, R>()), smem, s, TP, r, z, coarse_inv, coarse_invT);
+    SBM_PDL((k_vcycle_tail_cta<2, R>), 1, kTailCtaThreads, smem, s, TP, r, z, coarse_inv);
   else
-    SBM_PDL((k_vcycle_tail_cta<3, R>), 1, (tail_cta_threads<3, R>()), smem, s, TP, r, z, coarse_inv, coarse_invT);
+    SBM_PDL((k_vcycle_tail_cta<3, R>), 1, kTailCtaThreads, smem, s, TP, r, z, coarse_inv);
   count_launches();
   return cudaGetLastError();
 }
 template cudaError_t launch_vcycle_tail_cta<double>(int, const TailCta<double>&, const double*, double*,
-                                                    const double*, const void*, size_t, cudaStream_t);
+                                                    const double*, size_t, cudaStream_t);
 template cudaError_t launch_vcycle_tail_cta<float>(int, const TailCta<float>&, const float*, float*, const double*,
-                                                   const void*, size_t, cudaStream_t);
+                                                   size_t, cudaStream_t);
 
 template cudaError_t launch_vcycle_tail<double>(int, const TailLevel<double>*, int, const double*, double*,
                                                 const double*, int, int, int, const TailPlan&, cudaStream_t);

@@ -42,6 +42,7 @@ struct HostLevel {
   int colour_start[9] = {}, colour_nbnd[8] = {}, bstart[8] = {};
   std::vector<double> dhat;         // [n_bnd][nslot][dim][nq]  d / h (zero on non-surrogate slots)
   std::vector<double> binvT;        // [n_bnd][np][np]  (A_KK^{-1})^T: element (j, i) at j*np + i
+  std::vector<double> aselfT;       // [n_bnd][np][np] (A_KK)^T in the same form (p = 1 levels)
   std::vector<int> parent_code;     // [n_act] (parent compact index << 3) | child bits, or -1
   std::vector<int> children;        // [2^dim][n_act] compact index of child in the next finer level
   std::vector<int> sf_cell, sf_slot;
@@ -171,23 +172,34 @@ struct TailLevel {
   int ncell, zoff, roff;
 };
 
-// One-CTA V-cycle tail: the coarse p = 1 levels 0..top in a single CTA, with every level vector,
-// neighbour table, transfer table and boundary-cell inverse staged in its shared memory.  The
-// whole block is a kernel parameter (__grid_constant__), so every level constant is a constant-
-// bank read.  Offsets are in elements of R (vectors, inverses) or of int (tables).
+// One-CTA V-cycle tail: the coarse p = 1 levels 0..top in a single CTA, with every level vector and
+// table in its shared memory.  The tables are one image in global memory, laid out as they lie in shared
+// memory, [0, image_bytes): the level descriptors (TailLevelDesc, 0 first), their matrices, cell records,
+// child tables, boundary blocks and the coarse inverse.  The vectors follow.  Offsets in bytes.
+//
+// A level vector holds the cells' 16-byte words by plane: word w of cell a at (w * (n_act + 1) + a) * 16,
+// so that consecutive cells' words are adjacent (no bank conflicts); cell n_act stays zero and stands
+// for a missing neighbour.  Boundary blocks are padded by 16 bytes for the same reason.
 constexpr int kMaxTailCta = 6;
+constexpr int kTailMats = 136;     // coupling entries (8), interior inverse, interior block
+struct TailLevelDesc {
+  int n_act;
+  unsigned z, f, binv, aself, mats, rec, ch;   // aself 0: the boundary self blocks stay in global memory
+  // cell idx (0 <= idx < end2) of a colour group: idx + first0 below end0, + first1 below end1, + first2
+  // below end2 (a group has up to three colours, each a range of cells)
+  struct Group {
+    int end0, end1, end2, first0, first1, first2;
+  } grp[4];
+};
 template <typename R>
 struct TailCta {
-  int top, pre, post, ssor;
-  int zoff[kMaxTailCta], roff[kMaxTailCta], boff[kMaxTailCta];
-  int noff[kMaxTailCta], coff[kMaxTailCta], poff[kMaxTailCta];   // nbr, children, parent codes
-  int n_bnd[kMaxTailCta];
-  unsigned int_base;               // byte offset of the int area
-  int bulk;                        // 1: tables staged by bulk asynchronous copies (every table and
-                                   // its shared-memory slot 16-byte aligned), 0: by plain loads
-  unsigned cinv_off;               // byte offset of the staged FP64 coarse inverse, 0: read from global
-  LevelParams<R> P[kMaxTailCta];
-  TransferParams<R> T[kMaxTailCta];
+  int top, pre, post, ssor, n0;    // n0: unknowns of level 0
+  unsigned image_bytes, cinv;      // cinv: the coarse inverse's transpose in the image, 0: not staged
+  unsigned vec_bytes;              // the z vectors, from image_bytes on (the f vectors behind them)
+  const void* image;
+  const R* aselfT[kMaxTailCta];    // boundary self blocks in global memory, NP * NP each
+  R omega[kMaxTailCta];
+  R Ph[2][4];
 };
 
 // Launch shape of the cluster tail of one precision: cluster size (CTAs), dynamic shared

@@ -535,3 +535,26 @@ def test_device_geometry_matches_host(name, prob):
         assert np.abs(dd - dh).max(initial=0.0) <= 1e-12, (l, np.abs(dd - dh).max())
     gd.close()
     gh.close()
+
+
+@pytest.mark.parametrize("name,kw,offset", [
+    ("disk16", dict(), 0), ("disk16", dict(omega=0.8, ssor_each=1), 0), ("disk16", dict(pre_smooth=0, post_smooth=2), 1),
+    ("disk64", dict(coarsest_n=16), 0), ("star64", dict(pre_smooth=2), 0), ("sphere8", dict(), 1),
+    ("sphere16", dict(omega=0.9, post_smooth=2), 0), ("sphere32", dict(), 0)])
+def test_cta_tail_matches_per_level_launches(name, kw, offset):
+    """The one-CTA tail against the per-level launches, both FP32: whole V-cycles inside the tail (vectors at
+    an odd offset too), a coarse inverse too large to stage, boundary self blocks in and out of shared
+    memory, omega, SSOR and step counts.  Bound: FP32 sums in another order, 2e-5 relative."""
+    import paper_2506_12899_gb300 as S
+    prob = {"disk16": W.disk2d_p1(16, 1), "disk64": W.disk2d_p1(64, 2), "star64": W.star2d_p2(64, 1).replace(p=1),
+            "sphere8": W.sphere3d(8, 1, 1), "sphere16": W.sphere3d(16, 1, 2), "sphere32": W.sphere3d(32, 1, 0)}[name].replace(**kw)
+    a, b = S.Solver(prob, "f32"), S.Solver(prob, "f32", tail_max_cells=-1)
+    n = a.n_dof()
+    r = torch.rand(n + 1, generator=torch.Generator(device="cuda").manual_seed(3), device="cuda")[offset:offset + n] - 0.5
+    z = torch.empty(n + 1, device="cuda")[offset:offset + n]
+    before = S.kernel_launches()
+    a.vcycle(r, z)
+    used = S.kernel_launches() - before
+    ref = b.vcycle(r.clone())
+    assert used < S.kernel_launches() - before - used                 # the tail ran
+    assert (z - ref).norm() <= 2e-5 * ref.norm()
