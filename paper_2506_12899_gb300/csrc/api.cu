@@ -592,6 +592,15 @@ Context* build_context(const sbm_setup_desc& d, bool device) {
     L.P64 = make_params<double>(L, L.dhat64, L.binv64);
     L.P32 = make_params<float>(L, L.dhat32, L.binv32);
     L.P64.ordering = L.P32.ordering = d.ordering;
+    if (cell_smoother(L.H.dim, L.H.p) && L.H.n_bnd > 0) {   // the inverses by entry (thread-per-cell smoothers)
+      const size_t ld = ((size_t)L.H.n_bnd + 31) / 32 * 32, nq = (size_t)L.H.np * L.H.np;
+      std::vector<double> bs(nq * ld, 0.0);
+      for (int b = 0; b < L.H.n_bnd; ++b)
+        for (size_t q = 0; q < nq; ++q) bs[q * ld + b] = L.H.binvT[b * nq + q];
+      L.P64.bnd_ld = L.P32.bnd_ld = (int)ld;
+      if (d.cell_kernel_min_cells >= 0) L.P32.binvS = C->upload(to_f32(bs));
+      if (d.cell_kernel_min_cells > 0) L.P64.binvS = C->upload(bs);
+    }
     if (&L == &C->lv.back()) {                     // Arnoldi operator in double-float
       std::vector<dfl> dh(L.H.dhat.size());
       for (size_t i = 0; i < dh.size(); ++i) dh[i] = dfl(L.H.dhat[i]);

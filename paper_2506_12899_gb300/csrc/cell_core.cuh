@@ -569,6 +569,16 @@ template <int D, int N1, typename R>
 __device__ __forceinline__ void block_solve(const LevelParams<R>& P, int bidx, R (&t)[CD<D, N1>::NP],
                                             R (&y)[CD<D, N1>::NP]) {
   constexpr int NP = CD<D, N1>::NP;
+  if (bidx >= 0 && P.binvS) {
+    const R* B = P.binvS + bidx;
+#pragma unroll
+    for (int i = 0; i < NP; ++i) y[i] = 0;
+#pragma unroll
+    for (int j = 0; j < NP; ++j)
+#pragma unroll
+      for (int i = 0; i < NP; ++i) y[i] += B[(size_t)(j * NP + i) * P.bnd_ld] * t[j];
+    return;
+  }
   block_solve_at<D, N1, R>(P, bidx >= 0 ? P.binvT + (size_t)bidx * NP * NP : nullptr, t, y);
 }
 

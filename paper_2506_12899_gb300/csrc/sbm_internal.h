@@ -125,6 +125,10 @@ struct LevelParams {
   const int* nbr;
   const R* dhat;
   const R* binvT;
+  // the same inverses by entry, entry q of boundary cell b at q * bnd_ld + b (thread-per-cell smoothers: the
+  // lanes of a warp read neighbouring words; null elsewhere)
+  const R* binvS;
+  int bnd_ld;
   // dense self blocks h^(d-2) A_KK of the boundary cells (Eqs. 10, 7), column j at bself_ld * b + np * j
   // (double-float operator of a 3D p = 1 finest level only; null elsewhere)
   const R* bself;
