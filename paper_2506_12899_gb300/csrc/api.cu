@@ -592,14 +592,19 @@ Context* build_context(const sbm_setup_desc& d, bool device) {
     L.P64 = make_params<double>(L, L.dhat64, L.binv64);
     L.P32 = make_params<float>(L, L.dhat32, L.binv32);
     L.P64.ordering = L.P32.ordering = d.ordering;
-    if (cell_smoother(L.H.dim, L.H.p) && L.H.n_bnd > 0) {   // the inverses by entry (thread-per-cell smoothers)
+    if (cell_smoother(L.H.dim, L.H.p) && L.H.n_bnd > 0) {   // the blocks by entry (thread-per-cell kernels)
       const size_t ld = ((size_t)L.H.n_bnd + 31) / 32 * 32, nq = (size_t)L.H.np * L.H.np;
-      std::vector<double> bs(nq * ld, 0.0);
-      for (int b = 0; b < L.H.n_bnd; ++b)
-        for (size_t q = 0; q < nq; ++q) bs[q * ld + b] = L.H.binvT[b * nq + q];
+      auto by_entry = [&](const std::vector<double>& blocks) {
+        std::vector<double> s(nq * ld, 0.0);
+        for (int b = 0; b < L.H.n_bnd; ++b)
+          for (size_t q = 0; q < nq; ++q) s[q * ld + b] = blocks[b * nq + q];
+        return s;
+      };
+      const std::vector<double> bs = by_entry(L.H.binvT);
       L.P64.bnd_ld = L.P32.bnd_ld = (int)ld;
       if (d.cell_kernel_min_cells >= 0) L.P32.binvS = C->upload(to_f32(bs));
       if (d.cell_kernel_min_cells > 0) L.P64.binvS = C->upload(bs);
+      if (d.cell_kernel_min_cells >= 0 && L.H.p == 1) L.P32.aselfS = C->upload(to_f32(by_entry(L.H.aselfT)));
     }
     if (&L == &C->lv.back()) {                     // Arnoldi operator in double-float
       std::vector<dfl> dh(L.H.dhat.size());
@@ -812,15 +817,15 @@ template <typename R>
 void ensure_work(Context& C) {
   const int pi = prec_index<R>();
   if (C.work_ready[pi]) return;
+  // one allocation for every level's vectors, each on a 256-byte boundary
+  const int nvec = C.desc.smoother == 0 ? 3 : (C.desc.smoother == 2 ? 5 : 4);
+  auto padded = [](const DevLevel& L) { return ((size_t)L.H.n_dof() + 63) / 64 * 64; };
+  size_t total = 0;
+  for (auto& L : C.lv) total += nvec * padded(L);
+  R* next = C.dalloc<R>(total);
   for (auto& L : C.lv) {
-    size_t N = L.H.n_dof();
-    L.z[pi] = C.dalloc<R>(N);
-    L.rhs[pi] = C.dalloc<R>(N);
-    L.res[pi] = C.dalloc<R>(N);
-    if (C.desc.smoother != 0) {
-      L.tmp[pi] = C.dalloc<R>(N);
-      if (C.desc.smoother == 2) L.dir[pi] = C.dalloc<R>(N);
-    }
+    void** slots[5] = {&L.z[pi], &L.rhs[pi], &L.res[pi], &L.tmp[pi], &L.dir[pi]};
+    for (int k = 0; k < nvec; ++k, next += padded(L)) *slots[k] = next;
   }
   // cluster tail: the highest candidate level whose vectors (levels 0..top) fit in the shared
   // memory of a resident cluster of 16, else 8, CTAs

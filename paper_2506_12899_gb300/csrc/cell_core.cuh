@@ -473,9 +473,13 @@ __device__ __forceinline__ void load_nbr(const LevelParams<R>& P, int a, int (&n
 // weight times h^(d-2); a missing neighbour contributes zeros.  This executes about a quarter
 // fewer FP32 instructions than the face-by-face form.  FP32 and FP64 keep the face-by-face form,
 // which holds one neighbour at a time in registers.
-template <int D, int N1, typename TI, typename R>
+//
+// pre: h^(d-2) A_KK of a boundary cell in registers (NPRE = NP * NP entries), read before the dependency wait;
+// without it (NPRE = 1) the surrogate-face terms are evaluated.
+template <int D, int N1, typename TI, typename R, int NPRE = 1>
 __device__ __forceinline__ void cell_apply(const LevelParams<R>& P, const TI* __restrict__ x, int a,
-                                           const int (&nb)[2 * D], R (&y)[CD<D, N1>::NP]) {
+                                           const int (&nb)[2 * D], R (&y)[CD<D, N1>::NP],
+                                           const R (*pre)[NPRE] = nullptr) {
   constexpr int NP = CD<D, N1>::NP, NQ = CD<D, N1>::NQ;
   const LevelConsts<R>& C = P.k;
   if constexpr (std::is_same<R, dfl>::value && std::is_same<TI, float>::value) {
@@ -551,10 +555,18 @@ __device__ __forceinline__ void cell_apply(const LevelParams<R>& P, const TI* __
     load_cell<D, N1, TI, R>(x, a, P.n_act, v);
 #pragma unroll
     for (int i = 0; i < NP; ++i) y[i] = 0;
-    add_self<D, N1, R>(P, nb, boundary_index(P, a, 1 << D), v, y);
+    const int bidx = boundary_index(P, a, 1 << D);
+    const bool dense = NPRE > 1 && bidx >= 0;
+    if (!dense) add_self<D, N1, R>(P, nb, bidx, v, y);
     add_couplings<D, N1, TI, R>(P, x, 0, false, nb, y);
 #pragma unroll
     for (int i = 0; i < NP; ++i) y[i] *= P.hscale;
+    if (dense) {
+#pragma unroll
+      for (int j = 0; j < NP; ++j)
+#pragma unroll
+        for (int i = 0; i < NP; ++i) y[i] += (*pre)[NPRE > 1 ? j * NP + i : 0] * v[j];
+    }
   }
 }
 

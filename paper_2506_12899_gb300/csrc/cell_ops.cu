@@ -89,6 +89,24 @@ __global__ void __launch_bounds__(kCellThreads, 6) k_apply_cell_occ(const __grid
 }
 
 
+// The NN entries of boundary cell b's block stored by entry (LevelParams::binvS, aselfS); nothing if b < 0.
+template <int NN, typename R>
+__device__ __forceinline__ void load_block(const R* __restrict__ S, int ld, int b, R (&B)[NN]) {
+  if (b < 0) return;
+#pragma unroll
+  for (int q = 0; q < NN; ++q) B[q] = __ldg(S + (size_t)q * ld + b);
+}
+// y = B t, B by columns (never called with NN != NP * NP).
+template <int NP, int NN, typename R>
+__device__ __forceinline__ void dense_apply(const R (&B)[NN], const R (&t)[NP], R (&y)[NP]) {
+#pragma unroll
+  for (int i = 0; i < NP; ++i) y[i] = 0;
+#pragma unroll
+  for (int j = 0; j < NP; ++j)
+#pragma unroll
+    for (int i = 0; i < NP; ++i) y[i] += B[NN > 1 ? j * NP + i : 0] * t[j];
+}
+
 // One colour group of the block Gauss-Seidel sweep, one thread per cell: block b updates cells of
 // the segment whose block range holds b.
 //
@@ -118,12 +136,7 @@ __global__ void __launch_bounds__(PRE ? 32 : kCellThreads) k_smooth_cell(const _
   if (valid) {
     load_nbr<D, R>(P, a, nb);                        // set-up data: read before the wait
     if (early) load_cell_l2<D, N1, R, R>(f, a, P.n_act, t);   // f written two or more launches back
-    if constexpr (PRE) {
-      if (bidx >= 0) {
-#pragma unroll
-        for (int q = 0; q < NP * NP; ++q) B[q] = __ldg(P.binvS + (size_t)q * P.bnd_ld + bidx);
-      }
-    }
+    if constexpr (PRE) load_block(P.binvS, P.bnd_ld, bidx, B);
   }
   pdl_wait();
   pdl_trigger();
@@ -131,16 +144,8 @@ __global__ void __launch_bounds__(PRE ? 32 : kCellThreads) k_smooth_cell(const _
   if (valid) {
     if (!early) load_cell<D, N1, R, R>(f, a, P.n_act, t);
     smooth_rhs<D, N1, R>(P, G.col[sg], zero_start, nb, t, u);
-    if (PRE && bidx >= 0) {
-#pragma unroll
-      for (int i = 0; i < NP; ++i) y[i] = 0;
-#pragma unroll
-      for (int j = 0; j < NP; ++j)
-#pragma unroll
-        for (int i = 0; i < NP; ++i) y[i] += B[PRE ? j * NP + i : 0] * t[j];
-    } else {
-      block_solve<D, N1, R>(P, bidx, t, y);
-    }
+    if (PRE && bidx >= 0) dense_apply(B, t, y);
+    else block_solve<D, N1, R>(P, bidx, t, y);
     smooth_relax<D, N1, R>(P, zero_start, a, u, y);
   }
   if constexpr (cell_vec16<NP, R>()) {
@@ -221,8 +226,13 @@ __device__ __forceinline__ R h_weight(const TransferParams<R>& T, int o, int i, 
 // child's residual in registers, its restriction, then a fixed butterfly sum over the group.
 // SM0: also the first colour group of the coarse level's first pre-smoothing sweep from zero (see
 // k_resid_restrict_p_cell), computed by lane 0 of each coarse cell's group.
-template <int D, typename R, bool SM0>
-__global__ void __launch_bounds__(kCellThreads) k_resid_restrict_h_cell(const __grid_constant__ LevelParams<R> P,
+//
+// PRE (as in k_smooth_cell): the children's self blocks, instead of their surrogate-face terms, and with SM0 the
+// coarse cells' inverses are read before the dependency wait: V-cycle of the 64^3 p = 1 sphere 79.0 -> 77.2 us.
+// (Not at 2D p = 2, k_resid_restrict_p_cell: 81 registers of block made that V-cycle 1.8 us longer; nor after the
+// wait in the operator: 44 -> 46 us at 2048^2 p = 2.)
+template <int D, typename R, bool SM0, bool PRE>
+__global__ void __launch_bounds__(PRE ? 32 : kCellThreads) k_resid_restrict_h_cell(const __grid_constant__ LevelParams<R> P,
                                                                         const __grid_constant__ TransferParams<R> T,
                                                                         const R* __restrict__ u,
                                                                         const R* __restrict__ f, R* __restrict__ rc,
@@ -239,16 +249,21 @@ __global__ void __launch_bounds__(kCellThreads) k_resid_restrict_h_cell(const __
   const int a = cc < T.n_act_c ? T.children[(size_t)o * T.n_act_c + cc] : -1;
   int nb[2 * D];
   R fa[NP];
+  constexpr int NPRE = PRE ? NP * NP : 1, NPRC = PRE && SM0 ? NP * NP : 1;
+  R A[NPRE], B[NPRC];
   if (a >= 0) {
     load_nbr<D, R>(P, a, nb);
     if (early) load_cell_l2<D, 2, R, R>(f, a, P.n_act, fa);   // f written two or more launches back
+    if constexpr (PRE) load_block<NPRE>(P.aselfS, P.bnd_ld, boundary_index(P, a, 1 << D), A);
   }
+  if constexpr (PRE && SM0)
+    load_block<NPRC>(Pc.binvS, Pc.bnd_ld, o == 0 && cc < T.n_act_c && cc < Pc.colour_nbnd[0] ? Pc.bstart[0] + cc : -1, B);
   pdl_wait();
   pdl_trigger();
   if (a >= 0) {
     R r[NP];
     if (!early) load_cell<D, 2, R, R>(f, a, P.n_act, fa);
-    cell_apply<D, 2, R, R>(P, u, a, nb, r);
+    cell_apply<D, 2, R, R, NPRE>(P, u, a, nb, r, &A);
 #pragma unroll
     for (int i = 0; i < NP; ++i) r[i] = fa[i] - r[i];
 #pragma unroll
@@ -269,7 +284,9 @@ __global__ void __launch_bounds__(kCellThreads) k_resid_restrict_h_cell(const __
     if constexpr (SM0) {
       if (cc < Pc.colour_start[1]) {
         R y[NP];
-        block_solve<D, 2, R>(Pc, cc < Pc.colour_nbnd[0] ? Pc.bstart[0] + cc : -1, out, y);
+        const int bc = cc < Pc.colour_nbnd[0] ? Pc.bstart[0] + cc : -1;
+        if (PRE && bc >= 0) dense_apply<NP, NPRC>(B, out, y);
+        else block_solve<D, 2, R>(Pc, bc, out, y);
 #pragma unroll
         for (int j = 0; j < NP; ++j) y[j] = Pc.omega == R(1) ? y[j] : Pc.omega * y[j];
         store_cell<D, 2, R>(zc, cc, y);
@@ -919,15 +936,19 @@ cudaError_t launch_resid_restrict_h_cell(int dim, const LevelParams<R>& P, const
   const unsigned bs = cell_block((size_t)T.n_act_c << dim), g = cdiv((size_t)T.n_act_c << dim, bs);
   const bool sm0 = Pc != nullptr && zc != nullptr;
   const LevelParams<R>& Q = sm0 ? *Pc : P;
-  if (dim == 2) {
-    if (sm0) SBM_PDL((k_resid_restrict_h_cell<2, R, true>), g, bs, 0, s, P, T, u, f, rc, early, Q, zc);
-    else SBM_PDL((k_resid_restrict_h_cell<2, R, false>), g, bs, 0, s, P, T, u, f, rc, early, Q, zc);
-  } else if (dim == 3) {
-    if (sm0) SBM_PDL((k_resid_restrict_h_cell<3, R, true>), g, bs, 0, s, P, T, u, f, rc, early, Q, zc);
-    else SBM_PDL((k_resid_restrict_h_cell<3, R, false>), g, bs, 0, s, P, T, u, f, rc, early, Q, zc);
-  } else {
-    return cudaErrorInvalidValue;
+  constexpr bool kPre = sizeof(R) == 4;
+  const bool pre = kPre && bs == 32 && P.aselfS && (!sm0 || Q.binvS);
+#define SBM_RRHC(D)                                                                                               \
+  {                                                                                                               \
+    if (sm0 && pre) SBM_PDL((k_resid_restrict_h_cell<D, R, true, kPre>), g, bs, 0, s, P, T, u, f, rc, early, Q, zc); \
+    else if (sm0) SBM_PDL((k_resid_restrict_h_cell<D, R, true, false>), g, bs, 0, s, P, T, u, f, rc, early, Q, zc);  \
+    else if (pre) SBM_PDL((k_resid_restrict_h_cell<D, R, false, kPre>), g, bs, 0, s, P, T, u, f, rc, early, Q, zc);  \
+    else SBM_PDL((k_resid_restrict_h_cell<D, R, false, false>), g, bs, 0, s, P, T, u, f, rc, early, Q, zc);          \
   }
+  if (dim == 2) SBM_RRHC(2)
+  else if (dim == 3) SBM_RRHC(3)
+  else return cudaErrorInvalidValue;
+#undef SBM_RRHC
   count_launches();
   return cudaGetLastError();
 }

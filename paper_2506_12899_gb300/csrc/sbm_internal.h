@@ -42,7 +42,7 @@ struct HostLevel {
   int colour_start[9] = {}, colour_nbnd[8] = {}, bstart[8] = {};
   std::vector<double> dhat;         // [n_bnd][nslot][dim][nq]  d / h (zero on non-surrogate slots)
   std::vector<double> binvT;        // [n_bnd][np][np]  (A_KK^{-1})^T: element (j, i) at j*np + i
-  std::vector<double> aselfT;       // [n_bnd][np][np] (A_KK)^T in the same form (p = 1 levels)
+  std::vector<double> aselfT;       // [n_bnd][np][np] (A_KK)^T in the same form (levels with np <= 27)
   std::vector<int> parent_code;     // [n_act] (parent compact index << 3) | child bits, or -1
   std::vector<int> children;        // [2^dim][n_act] compact index of child in the next finer level
   std::vector<int> sf_cell, sf_slot;
@@ -128,6 +128,9 @@ struct LevelParams {
   // the same inverses by entry, entry q of boundary cell b at q * bnd_ld + b (thread-per-cell smoothers: the
   // lanes of a warp read neighbouring words; null elsewhere)
   const R* binvS;
+  // h^(d-2) A_KK of the boundary cells by entry in the same way, column j row i at entry j * np + i
+  // (FP32 p = 1 levels: k_resid_restrict_h_cell; null elsewhere)
+  const R* aselfS;
   int bnd_ld;
   // dense self blocks h^(d-2) A_KK of the boundary cells (Eqs. 10, 7), column j at bself_ld * b + np * j
   // (double-float operator of a 3D p = 1 finest level only; null elsewhere)

@@ -695,7 +695,8 @@ HostLevel build_level(const sbm_setup_desc& d, int n, int p, bool device, std::v
 
   // dense blocks A_KK of boundary cells (Eq. 14) and their inverses, stored transposed
   L.binvT.assign((size_t)L.n_bnd * np * np, 0.0);
-  if (p == 1) L.aselfT.assign((size_t)L.n_bnd * np * np, 0.0);
+  const bool keep_self = np <= 27;
+  if (keep_self) L.aselfT.assign((size_t)L.n_bnd * np * np, 0.0);
   std::vector<double> ratio(L.n_bnd, 1.0);
   parallel_for(L.n_bnd, [&](int b0, int b1) {
     std::vector<double> A((size_t)np * np), inv, e(np), col(np);
@@ -706,7 +707,7 @@ HostLevel build_level(const sbm_setup_desc& d, int n, int p, bool device, std::v
         e[j] = 1.0;
         cell_self_apply(L, a, b, e.data(), col.data());
         for (int i = 0; i < np; ++i) A[(size_t)i * np + j] = col[i];
-        if (p == 1) std::copy(col.begin(), col.end(), &L.aselfT[((size_t)b * np + j) * np]);
+        if (keep_self) std::copy(col.begin(), col.end(), &L.aselfT[((size_t)b * np + j) * np]);
       }
       ratio[b] = dense_inverse(np, A, inv);
       for (int i = 0; i < np; ++i)
