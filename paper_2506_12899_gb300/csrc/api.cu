@@ -592,6 +592,7 @@ Context* build_context(const sbm_setup_desc& d, bool device) {
     L.P64 = make_params<double>(L, L.dhat64, L.binv64);
     L.P32 = make_params<float>(L, L.dhat32, L.binv32);
     L.P64.ordering = L.P32.ordering = d.ordering;
+    if (!L.H.aselfT.empty()) L.P64.aselfT = C->upload(L.H.aselfT);
     if (cell_smoother(L.H.dim, L.H.p) && L.H.n_bnd > 0) {   // the blocks by entry (thread-per-cell kernels)
       const size_t ld = ((size_t)L.H.n_bnd + 31) / 32 * 32, nq = (size_t)L.H.np * L.H.np;
       auto by_entry = [&](const std::vector<double>& blocks) {

@@ -189,17 +189,26 @@ __device__ __forceinline__ R apply_dof(const LevelParams<R>& P, const LevelConst
   int ii[3];
   decompose<D, N1>(i, ii);
   R acc = 0;
+  const int bidx = valid ? bnd_index(P, a, 1 << D) : -1;
+  // A boundary cell with a stored self block applies that: np FMAs per value on full warps, where the
+  // surrogate-face terms take 2d barrier-separated phases in which one thread in N1 works (on the
+  // FP64 pipe an idle lane costs as much as a busy one).  64^3 p = 2 sphere in FP64, with
+  // the restriction by directions below: residual + p-restriction 230 -> 110 us, the four residual +
+  // h-restrictions 138 -> 59.
+  const bool dense = bidx >= 0 && P.aselfT != nullptr;
   if (valid) {
 #pragma unroll
     for (int dir = 0; dir < D; ++dir) {
       const int st = stride_of<N1>(dir), id = ii[dir], base = i - id * st;
       R wt;
       tang<D, N1>(ii, dir, C.w, wt);
-      const int mask = (nb[2 * dir] >= 0) + 2 * (nb[2 * dir + 1] >= 0);
-      const R* Lm = C.L[mask];
       R s = 0;
+      if (!dense) {
+        const int mask = (nb[2 * dir] >= 0) + 2 * (nb[2 * dir + 1] >= 0);
+        const R* Lm = C.L[mask];
 #pragma unroll
-      for (int k = 0; k < N1; ++k) s += Lm[id * N1 + k] * sU[c * NP + base + k * st];
+        for (int k = 0; k < N1; ++k) s += Lm[id * N1 + k] * sU[c * NP + base + k * st];
+      }
       if (nb[2 * dir] >= 0) {
 #pragma unroll
         for (int k = 0; k < N1; ++k) s += C.Bpm[id * N1 + k] * sN[(c * NS + 2 * dir) * NP + base + k * st];
@@ -211,7 +220,15 @@ __device__ __forceinline__ R apply_dof(const LevelParams<R>& P, const LevelConst
       acc += wt * s;
     }
   }
-  const int bidx = valid ? bnd_index(P, a, 1 << D) : -1;
+  if (P.aselfT != nullptr) {
+    acc *= P.hscale;
+    if (dense) {
+      const R* A = P.aselfT + (size_t)bidx * NP * NP + i;
+#pragma unroll
+      for (int j = 0; j < NP; ++j) acc += A[(size_t)j * NP] * sU[c * NP + j];
+    }
+    return acc;
+  }
   unsigned smask = 0;                               // bit s: face slot s is a surrogate face
 #pragma unroll
   for (int s = 0; s < NS; ++s) smask |= (nb[s] < 0 ? 1u : 0u) << s;
@@ -275,23 +292,30 @@ __global__ void __launch_bounds__(256) k_resid_restrict_p(const __grid_constant_
   __syncthreads();                                   // sU is reused for the residual
   sU[c * NP + i] = valid ? fv - v : R(0);
   __syncthreads();
-  if (valid && i < NPC) {
-    const int j0 = i % NC, j1 = (i / NC) % NC, j2 = D == 3 ? i / (NC * NC) : 0;
-    const R* r = sU + c * NP;
-    R s2 = 0;
+  // one direction at a time (N1 -> NC values), each by as many threads as it has results
+  constexpr int NX = NPC / NC * N1, NXX = D == 3 ? NC * N1 * N1 : NX;   // results after (x and) all but the last
+  R* src = sU;                                       // and after x alone
+  R* dst = sN;
 #pragma unroll
-    for (int i2 = 0; i2 < (D == 3 ? N1 : 1); ++i2) {
-      R s1 = 0;
+  for (int dir = 0; dir < D; ++dir) {
+    constexpr int kCnt[3] = {NXX, D == 3 ? NX : NPC, NPC};
+    const int cnt = kCnt[dir], lo = dir == 0 ? 1 : (dir == 1 ? NC : NC * NC);   // results below: lo per step of dir
+    if (i < cnt) {
+      const int low = i % lo, jd = (i / lo) % NC, high = i / (lo * NC);
+      const R* r = src + c * NP + low + high * lo * N1;
+      R v = 0;
 #pragma unroll
-      for (int i1 = 0; i1 < N1; ++i1) {
-        R s0 = 0;
-#pragma unroll
-        for (int i0 = 0; i0 < N1; ++i0) s0 += sPp[i0 * NC + j0] * r[i0 + N1 * i1 + N1 * N1 * i2];
-        s1 += sPp[i1 * NC + j1] * s0;
+      for (int q = 0; q < N1; ++q) v += sPp[q * NC + jd] * r[q * lo];
+      if (dir == D - 1) {
+        if (valid) rc[(size_t)a * NPC + i] = v;
+      } else {
+        dst[c * NP + i] = v;
       }
-      s2 += (D == 3 ? sPp[i2 * NC + j2] : R(1)) * s1;
     }
-    rc[(size_t)a * NPC + i] = s2;
+    if (dir < D - 1) __syncthreads();
+    R* tmp = src;
+    src = dst;
+    dst = tmp;
   }
 }
 
@@ -329,32 +353,28 @@ __global__ void __launch_bounds__(256) k_resid_restrict_h(const __grid_constant_
   __syncthreads();                                   // sU is reused for the residuals
   sU[c * NP + i] = valid ? fv - v : R(0);
   __syncthreads();
+  // every child restricts its own residual, one direction at a time; then a sum over the children
+  R* src = sU;
+  R* dst = sN;
+#pragma unroll
+  for (int dir = 0; dir < D; ++dir) {
+    const int lo = 1 << dir, jd = (i >> dir) & 1;
+    const R* P1 = sPh[(o >> dir) & 1];
+    const R* r = src + c * NP + (i & ~lo);
+    dst[c * NP + i] = P1[jd] * r[0] + P1[2 + jd] * r[lo];
+    __syncthreads();
+    R* tmp = src;
+    src = dst;
+    dst = tmp;
+  }
   const int t = threadIdx.x;
   if (t < CPC * NP) {                               // coarse dof j of coarse cell t / NP (NPC = NP for p = 1)
     const int ccl = t / NP, j = t % NP;
     const int cc2 = blockIdx.x * CPC + ccl;
     if (cc2 < T.n_act_c) {
-      const int j0 = j & 1, j1 = (j >> 1) & 1, j2 = (j >> 2) & 1;
       R sum = 0;
 #pragma unroll
-      for (int oo = 0; oo < NCH; ++oo) {
-        const R* r = sU + (ccl * NCH + oo) * NP;
-        const R* P0 = sPh[oo & 1];
-        const R* P1 = sPh[(oo >> 1) & 1];
-        const R* P2 = sPh[(oo >> 2) & 1];
-        R s2 = 0;
-#pragma unroll
-        for (int i2 = 0; i2 < (D == 3 ? 2 : 1); ++i2) {
-          R s1 = 0;
-#pragma unroll
-          for (int i1 = 0; i1 < 2; ++i1) {
-            const R s0 = P0[0 * 2 + j0] * r[0 + 2 * i1 + 4 * i2] + P0[1 * 2 + j0] * r[1 + 2 * i1 + 4 * i2];
-            s1 += P1[i1 * 2 + j1] * s0;
-          }
-          s2 += (D == 3 ? P2[i2 * 2 + j2] : R(1)) * s1;
-        }
-        sum += s2;
-      }
+      for (int oo = 0; oo < NCH; ++oo) sum += src[(ccl * NCH + oo) * NP + j];
       rc[(size_t)cc2 * NP + j] = sum;
     }
   }
@@ -570,6 +590,52 @@ __global__ void __launch_bounds__(256) k_prolong(const __grid_constant__ Transfe
     s2 += (D == 3 ? P2[i2 * NC + j2] : R(1)) * s1;
   }
   uf[(size_t)a * NPF + i] = uv + s2;
+}
+
+// The p-prolongation (same mesh, degree NC - 1 -> NF - 1) one direction at a time through shared memory, one
+// thread per fine value, a block of CPB cells: NC multiply-adds and reads per direction instead of NC^d of
+// each (64^3 p = 2 in FP64, bound by its pipe: 37 -> 20 us; 96^3 p = 3 in FP32, bound by the reads: the solve 85.7 ->
+// 83.2 ms).
+template <int D, int NF, int NC, typename R>
+__global__ void __launch_bounds__(256) k_prolong_p(const __grid_constant__ TransferParams<R> T,
+                                                   const R* __restrict__ ec, R* __restrict__ uf, int early) {
+  constexpr int NPF = D == 2 ? NF * NF : NF * NF * NF;
+  constexpr int NPC = D == 2 ? NC * NC : NC * NC * NC;
+  constexpr int CPB = 256 / NPF;
+  __shared__ R sA[CPB * NPF], sB[CPB * NPF], sPp[NF * NC];
+  const int c = threadIdx.x / NPF, i = threadIdx.x - c * NPF;
+  const int a0 = blockIdx.x * CPB, a = a0 + c;
+  const bool valid = a < T.n_act_f;
+  if (threadIdx.x < NF * NC) sPp[threadIdx.x] = T.Pp[threadIdx.x];
+  R uv = 0;
+  if (early && valid) uv = __ldcg(uf + (size_t)a * NPF + i);   // uf two launches back (L2)
+  pdl_wait();
+  pdl_trigger();
+  if (!early && valid) uv = uf[(size_t)a * NPF + i];
+  const int ncell = min(CPB, T.n_act_f - a0);
+  for (int q = threadIdx.x; q < ncell * NPC; q += CPB * NPF) sA[q / NPC * NPF + q % NPC] = ec[(size_t)a0 * NPC + q];
+  __syncthreads();
+  R* src = sA;
+  R* dst = sB;
+  R v = 0;
+#pragma unroll
+  for (int dir = 0; dir < D; ++dir) {
+    constexpr int kCnt[3] = {NF * NPC / NC, D == 3 ? NF * NF * NC : NPF, NPF};
+    const int lo = dir == 0 ? 1 : (dir == 1 ? NF : NF * NF);
+    if (i < kCnt[dir]) {
+      const int low = i % lo, id = (i / lo) % NF, high = i / (lo * NF);
+      const R* e = src + c * NPF + low + high * lo * NC;
+      v = 0;
+#pragma unroll
+      for (int q = 0; q < NC; ++q) v += sPp[id * NC + q] * e[q * lo];
+      if (dir < D - 1) dst[c * NPF + i] = v;
+    }
+    if (dir < D - 1) __syncthreads();
+    R* tmp = src;
+    src = dst;
+    dst = tmp;
+  }
+  if (valid) uf[(size_t)a * NPF + i] = uv + v;
 }
 
 // e = Ainv r in FP64; one warp per row.
@@ -806,7 +872,11 @@ cudaError_t launch_prolong(int dim, int pf, int pc, const TransferParams<R>& T, 
                            int early) {
   if (T.n_act_f == 0) return cudaSuccess;
 #define SBM_PROLONG(D, NF, NC)                                                    \
-  {                                                                               \
+  if constexpr (NF != NC) {                                                       \
+    constexpr int kNpf = D == 2 ? NF * NF : NF * NF * NF, kCpb = 256 / kNpf;      \
+    SBM_PDL((k_prolong_p<D, NF, NC, R>), ceil_div(T.n_act_f, kCpb), kCpb * kNpf, 0, s, T, ec, uf, early); \
+    count_launches();                                                             \
+  } else {                                                                        \
     const size_t n = (size_t)T.n_act_f * (D == 2 ? NF * NF : NF * NF * NF);       \
     SBM_PDL((k_prolong<D, NF, NC, R>), ceil_div(n, 256), 256, 0, s, T, ec, uf, early);   \
     count_launches();                                                             \

@@ -132,6 +132,9 @@ struct LevelParams {
   // (FP32 p = 1 levels: k_resid_restrict_h_cell; null elsewhere)
   const R* aselfS;
   int bnd_ld;
+  // h^(d-2) A_KK of the boundary cells, transposed, block b at b * np * np (FP64 levels with np <= 27; null elsewhere:
+  // the thread-per-DoF kernels then evaluate the surrogate-face terms)
+  const R* aselfT;
   // dense self blocks h^(d-2) A_KK of the boundary cells (Eqs. 10, 7), column j at bself_ld * b + np * j
   // (double-float operator of a 3D p = 1 finest level only; null elsewhere)
   const R* bself;
