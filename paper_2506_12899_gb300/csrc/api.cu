@@ -293,6 +293,7 @@ struct Context {
   double* v64 = nullptr;             // FP64 copy of v_j for the FP64 V-cycle on a double-float basis
   int ws_basis = -1;
   double* partial = nullptr;
+  double* partial2 = nullptr;      // partial sums of the second Gram-Schmidt sweep
   double* dots = nullptr;          // [0,32) h1, [32,64) h2, [64] norm, [96, 128) Hessenberg column
   double* ydev = nullptr;
   double* bbuf = nullptr;
@@ -309,7 +310,8 @@ struct Context {
   double* gsw = nullptr;           // [ldv] w, FP64
   float2* gswdf = nullptr;         // [ldv] w, double-float
   double* gspartial = nullptr;
-  double* gsdots = nullptr;        // [0,32) h1, [32,64) h2, [64] |w|, [65] 1.0, [128,161) column
+  double* gspartial2 = nullptr;
+  double* gsdots = nullptr;        // [0,32) h1, [32,64) h2, [64] |w|, [65] 1.0
   // sbm_l2_error: background indices of the finest cells, partial sums, result
   int* l2cell = nullptr;
   double* l2partial = nullptr;
@@ -1076,6 +1078,7 @@ void ensure_krylov(Context& C, int m) {
   C.w = C.dalloc<double>(C.ldv);
   if (prec == SBM_F32) C.r32 = C.dalloc<float>(N);
   C.partial = C.dalloc<double>((size_t)std::max(dot_blocks(N), gs_blocks(N)) * 32);   // rows of either grid
+  C.partial2 = C.dalloc<double>((size_t)gs_blocks(N) * 32);
   C.dots = C.dalloc<double>(128);
   C.ydev = C.dalloc<double>(32);
   C.ws_m = m;
@@ -1131,22 +1134,26 @@ void arnoldi_step_work(Context& C, int j, cudaStream_t s) {
         dfl* wd = reinterpret_cast<dfl*>(C.wdf);
         if (cell_smoother(dim, p)) CUDA_TRY((launch_apply_cell<float, dfl>(dim, p, F.Pdf, Zj, nullptr, wd, 0, s)));
         else CUDA_TRY((launch_apply<float, dfl>(dim, p, F.Pdf, Zj, nullptr, wd, 0, s)));   // one thread per DoF
-        CUDA_TRY(launch_gs_dot_df(C.V2, C.ldv, j + 1, C.wdf, N, C.partial, h1, s));
+        CUDA_TRY(launch_gs_dot_df(C.V2, C.ldv, j + 1, C.wdf, N, C.partial, s));
       } else {
         CUDA_TRY((launch_apply<float, double>(dim, p, F.P64, Zj, nullptr, C.w, 0, s)));
-        CUDA_TRY(launch_gs_dot(C.V2, C.ldv, j + 1, C.w, C.wdf, N, C.partial, h1, s));
+        CUDA_TRY(launch_gs_dot(C.V2, C.ldv, j + 1, C.w, C.wdf, N, C.partial, s));
       }
     } else {
       double* Zj = static_cast<double*>(C.Z) + (size_t)j * N;
       vcycle_rec<double>(C, Lf, C.v64, Zj, s);
       CUDA_TRY((launch_apply<double, double>(dim, p, F.P64, Zj, nullptr, C.w, 0, s)));
-      CUDA_TRY(launch_gs_dot(C.V2, C.ldv, j + 1, C.w, C.wdf, N, C.partial, h1, s));
+      CUDA_TRY(launch_gs_dot(C.V2, C.ldv, j + 1, C.w, C.wdf, N, C.partial, s));
     }
-    CUDA_TRY(launch_gs_axpy_dot(C.V2, C.ldv, j + 1, h1, C.wdf, N, C.partial, h2, s));
-    CUDA_TRY(launch_gs_axpy_norm(C.V2, C.ldv, j + 1, h2, C.wdf, N, C.partial, hn, s, h1, col));   // + column
+    // the partial sums alternate between two buffers: a sweep reads those of the sweep before
+    int nblk = 1;
+    CUDA_TRY(launch_gs_axpy_dot(C.V2, C.ldv, j + 1, C.partial, h1, C.wdf, N, C.partial2, s));
+    CUDA_TRY(launch_gs_axpy_norm(C.V2, C.ldv, j + 1, C.partial2, h2, C.wdf, N, C.partial, &nblk, s));
     float2* vnext = C.V2 + (size_t)(j + 1) * C.ldv;
-    if (prec == SBM_F32) CUDA_TRY((launch_gs_scale<float2, float>(C.wdf, hn, vnext, C.r32, N, s)));
-    else CUDA_TRY((launch_gs_scale<float2, double>(C.wdf, hn, vnext, C.v64, N, s)));
+    if (prec == SBM_F32)
+      CUDA_TRY(launch_gs_scale_norm<float>(C.wdf, C.partial, nblk, hn, h1, h2, j + 1, col, vnext, C.r32, N, s));
+    else
+      CUDA_TRY(launch_gs_scale_norm<double>(C.wdf, C.partial, nblk, hn, h1, h2, j + 1, col, vnext, C.v64, N, s));
   }
   if (C.desc.krylov_basis == 1) CUDA_TRY(launch_hess_column(h1, h2, hn, j + 1, col, s));
   CUDA_TRY(cudaMemcpyAsync(column_slot(C, j), col, (j + 2) * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1242,8 +1249,8 @@ int solve_impl(Context& C, const double* b, double* x, double tol, int m, int ma
         break;
       }
       if (C.desc.krylov_basis == 1) CUDA_TRY(launch_div_scalar(r0, hn, r0, N, s));
-      else if (prec == SBM_F32) CUDA_TRY((launch_gs_scale<double, float>(r0, hn, C.V2, C.r32, N, s)));
-      else CUDA_TRY((launch_gs_scale<double, double>(r0, hn, C.V2, C.v64, N, s)));
+      else if (prec == SBM_F32) CUDA_TRY((launch_gs_scale<float>(r0, hn, C.V2, C.r32, N, s)));
+      else CUDA_TRY((launch_gs_scale<double>(r0, hn, C.V2, C.v64, N, s)));
       std::fill(H.begin(), H.end(), 0.0);
       std::fill(g.begin(), g.end(), 0.0);
       g[0] = beta;
@@ -1764,6 +1771,7 @@ int sbm_gram_schmidt(void* ctx, int variant, const double* V_dev, int nv, const 
       C->gsw = C->dalloc<double>(ldv);
       C->gswdf = C->dalloc<float2>(ldv);
       C->gspartial = C->dalloc<double>((size_t)std::max(dot_blocks(N), gs_blocks(N)) * 32);
+      C->gspartial2 = C->dalloc<double>((size_t)gs_blocks(N) * 32);
       C->gsdots = C->dalloc<double>(256);
       const double one = 1.0;
       CUDA_TRY(cudaMemcpy(C->gsdots + 65, &one, sizeof(double), cudaMemcpyHostToDevice));
@@ -1773,7 +1781,6 @@ int sbm_gram_schmidt(void* ctx, int variant, const double* V_dev, int nv, const 
     double* h2 = C->gsdots + 32;
     double* hn = C->gsdots + 64;
     const double* one = C->gsdots + 65;
-    double* col = C->gsdots + 128;
     // w into the padded buffer (the staged copies read whole 16-byte units past an odd N)
     auto copy_w = [&] {
       CUDA_TRY(cudaMemsetAsync(C->gsw, 0, ldv * sizeof(double), s));
@@ -1791,20 +1798,22 @@ int sbm_gram_schmidt(void* ctx, int variant, const double* V_dev, int nv, const 
         CUDA_TRY(cudaMemsetAsync(C->gsV2, 0, 32 * ldv * sizeof(float2), s));
       }
       for (int k = 0; k < nv; ++k)                   // rows rounded to double-float (exact split)
-        CUDA_TRY((launch_gs_scale<double, double>(V_dev + (size_t)k * N, one, C->gsV2 + (size_t)k * ldv,
+        CUDA_TRY((launch_gs_scale<double>(V_dev + (size_t)k * N, one, C->gsV2 + (size_t)k * ldv,
                                                   (double*)nullptr, N, s)));
       // The sweeps read V before their dependency wait, so its last row must not come from the launch
       // just before them: the copies of w in between (no programmatic launch crosses a copy) see to that.
       copy_w();
       if (variant == 1) {                            // w handed over as double-float (FP32-V-cycle solves)
         CUDA_TRY(cudaMemsetAsync(C->gswdf, 0, ldv * sizeof(float2), s));
-        CUDA_TRY((launch_gs_scale<double, double>(C->gsw, one, C->gswdf, (double*)nullptr, N, s)));
-        CUDA_TRY(launch_gs_dot_df(C->gsV2, ldv, nv, C->gswdf, N, C->gspartial, h1, s));
+        CUDA_TRY((launch_gs_scale<double>(C->gsw, one, C->gswdf, (double*)nullptr, N, s)));
+        CUDA_TRY(launch_gs_dot_df(C->gsV2, ldv, nv, C->gswdf, N, C->gspartial, s));
       } else {                                       // w in FP64, converted by the first sweep
-        CUDA_TRY(launch_gs_dot(C->gsV2, ldv, nv, C->gsw, C->gswdf, N, C->gspartial, h1, s));
+        CUDA_TRY(launch_gs_dot(C->gsV2, ldv, nv, C->gsw, C->gswdf, N, C->gspartial, s));
       }
-      CUDA_TRY(launch_gs_axpy_dot(C->gsV2, ldv, nv, h1, C->gswdf, N, C->gspartial, h2, s));
-      CUDA_TRY(launch_gs_axpy_norm(C->gsV2, ldv, nv, h2, C->gswdf, N, C->gspartial, hn, s, h1, col));
+      int nblk = 1;
+      CUDA_TRY(launch_gs_axpy_dot(C->gsV2, ldv, nv, C->gspartial, h1, C->gswdf, N, C->gspartial2, s));
+      CUDA_TRY(launch_gs_axpy_norm(C->gsV2, ldv, nv, C->gspartial2, h2, C->gswdf, N, C->gspartial, &nblk, s));
+      CUDA_TRY(launch_gs_norm(C->gspartial, nblk, hn, s));
       CUDA_TRY(launch_df_to<double>(C->gswdf, w_out_dev, N, s));
     }
     CUDA_TRY(cudaMemcpyAsync(h_dev, h1, nv * sizeof(double), cudaMemcpyDeviceToDevice, s));

@@ -180,27 +180,6 @@ __global__ void k_cast(const TI* __restrict__ x, TO* __restrict__ y, size_t N) {
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += stride) y[i] = (TO)x[i];
 }
 
-// The norm sweep's reduction fused with the Hessenberg column: warp 0 sums the partial squares
-// (same order as k_reduce_partials) into hn[0] = |w| and col[k]; threads i < k write
-// col[i] = h1[i] + h2[i].
-__global__ void __launch_bounds__(64) k_reduce_norm_column(const double* __restrict__ partial, int nblk,
-                                                          double* __restrict__ hn, const double* __restrict__ h1,
-                                                          const double* __restrict__ h2, int k, double* __restrict__ col) {
-  pdl_entry();
-  const int i = threadIdx.x;
-  if (i < k) col[i] = h1[i] + h2[i];
-  if (i < 32) {
-    double s = 0.0;
-    for (int b = i; b < nblk; b += 32) s += partial[(size_t)b * kMaxVec];
-    s = warp_sum(s);
-    if (i == 0) {
-      const double r = sqrt(s);
-      hn[0] = r;
-      col[k] = r;
-    }
-  }
-}
-
 __global__ void k_hess_column(const double* h1, const double* h2, const double* hn, int k, double* col) {
   pdl_entry();
   const int i = threadIdx.x;
@@ -336,10 +315,13 @@ struct SweepShape {
 //         wdf as double-float for the next sweeps) or double-float (TW = float2).
 // MODE 1: wdf <- wdf - sum_k h[k] V_k, then partial[block][k] = V_k . wdf.
 // MODE 2: wdf <- wdf - sum_k h[k] V_k, then partial[block][0] = |wdf|^2.
+// MODE 1 and 2 take h as the partial sums hpart of the sweep before (the same grid): every block sums them
+// itself, in one fixed order, while its first copies of V are in flight, and block 0 writes h out.  (A
+// one-block launch for each reduction stood between the sweeps before: 512^2 p = 2 solve 6.02 -> 5.96 ms.)
 template <int NV, int MODE, typename TW>
 __global__ void __launch_bounds__(kSweepThreads) k_gs_sweep(const float2* __restrict__ V, size_t ldv, const TW* w_in,
-                                                            const double* __restrict__ h, float2* wdf, size_t N,
-                                                            double* __restrict__ partial) {
+                                                            const double* __restrict__ hpart, double* __restrict__ h,
+                                                            float2* wdf, size_t N, double* __restrict__ partial) {
   using Sh = SweepShape<NV>;
   constexpr int E = Sh::E, S = Sh::S, SLOT = Sh::SLOT, EPT = E / kSweepThreads;
   constexpr int NA = MODE == 2 ? 1 : NV;
@@ -374,23 +356,31 @@ __global__ void __launch_bounds__(kSweepThreads) k_gs_sweep(const float2* __rest
                 reinterpret_cast<const unsigned char*>(w_in) + e0 * sizeof(float2), bytes, &bar[q % S]);
     }
   };
-  // The first S chunks are copied before the dependency wait where that is safe: the V rows, and
-  // w for the update sweeps, were written at least two launches back, and this grid starts only
-  // after the kernel before it has passed its own griddepcontrol.wait, i.e. after everything
-  // before that kernel has completed and become visible.  h, and w of the dot sweep (the operator
-  // writes it just before), are read after the wait.
+  // The V rows of the first S chunks are copied before the dependency wait: they were written at
+  // least two launches back, and this grid starts only after the kernel before it has passed its
+  // own griddepcontrol.wait, i.e. after everything before that kernel has completed and become
+  // visible.  w and the partial sums come from the kernel just before and are read after the wait.
   if (tid == 0) {
     for (int q = 0; q < S; ++q) mbar_init(&bar[q], 1);
     mbar_fence_init();
-    for (size_t q = 0; q < (size_t)S && q < mine; ++q) {
-      issue_v(q);
-      if (MODE != 0) issue_w(q);
-    }
+    for (size_t q = 0; q < (size_t)S && q < mine; ++q) issue_v(q);
   }
   pdl_entry();
-  if (tid == 0 && MODE == 0)
+  if (tid == 0)
     for (size_t q = 0; q < (size_t)S && q < mine; ++q) issue_w(q);
-  if (MODE != 0 && tid < NV) hs[tid] = df_from_double(h[tid]);
+  if (MODE != 0) {
+    const int lane = tid & 31;
+#pragma unroll 1
+    for (int k = tid >> 5; k < NV; k += kSweepThreads / 32) {
+      double t = 0.0;
+      for (int b = lane; b < (int)gridDim.x; b += 32) t += hpart[(size_t)b * kMaxVec + k];
+      t = warp_sum(t);
+      if (lane == 0) {
+        hs[k] = df_from_double(t);
+        if (blockIdx.x == 0) h[k] = t;
+      }
+    }
+  }
   __syncthreads();
   float s[NA], c[NA];
 #pragma unroll
@@ -449,33 +439,58 @@ __global__ void __launch_bounds__(kSweepThreads) k_gs_sweep(const float2* __rest
   block_partials_df<NA>(s, c, partial);
 }
 
-// v = w / sc[0] as double-float (w FP64 or double-float), and, if out is not null, v rounded to
-// TO (the next V-cycle's input).
-template <typename TW, typename TO>
-__global__ void k_gs_scale(const TW* __restrict__ w, const double* __restrict__ sc, float2* __restrict__ v,
+// v = w / sc[0] as double-float, and, if out is not null, v rounded to TO (the next V-cycle's input).
+template <typename TO>
+__global__ void k_gs_scale(const double* __restrict__ w, const double* __restrict__ sc, float2* __restrict__ v,
                            TO* __restrict__ out, size_t N) {
   pdl_entry();
   const double inv = 1.0 / sc[0];
-  const float2 g = df_from_double(inv);
   const size_t stride = (size_t)gridDim.x * blockDim.x;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += stride) {
-    float2 r;
-    if constexpr (sizeof(TW) == 8 && std::is_same<TW, double>::value) {
-      r = df_from_double(w[i] * inv);
-    } else {                                        // double-float product, renormalised
-      const float2 a = w[i];
-      const float p = __fmul_rn(a.x, g.x);
-      float e = fmaf(a.x, g.x, -p);
-      e = fmaf(a.x, g.y, e);
-      e = fmaf(a.y, g.x, e);
-      const float hi = __fadd_rn(p, e);
-      r = make_float2(hi, __fsub_rn(e, __fsub_rn(hi, p)));
-    }
+    const float2 r = df_from_double(w[i] * inv);
     v[i] = r;
     if (out) {
       if constexpr (sizeof(TO) == 4) out[i] = __fadd_rn(r.x, r.y);
       else out[i] = df_to_double(r);
     }
+  }
+}
+
+// k_gs_scale after a MODE 2 sweep of nblk blocks: sc = |w| from its partial sums (every block sums them in the
+// same fixed order), block 0 also writes |w| and the Hessenberg column col[i] = h1[i] + h2[i] (i < k),
+// col[k] = |w|.
+template <typename TO>
+__global__ void __launch_bounds__(256) k_gs_scale_norm(const float2* __restrict__ w, const double* __restrict__ partial,
+                                                       int nblk, double* __restrict__ hn, const double* __restrict__ h1,
+                                                       const double* __restrict__ h2, int k, double* __restrict__ col,
+                                                       float2* __restrict__ v, TO* __restrict__ out, size_t N) {
+  __shared__ double norm;
+  pdl_entry();
+  if (threadIdx.x < 32) {
+    double s = 0.0;
+    for (int b = threadIdx.x; b < nblk; b += 32) s += partial[(size_t)b * kMaxVec];
+    s = warp_sum(s);
+    if (threadIdx.x == 0) norm = sqrt(s);
+  }
+  __syncthreads();
+  if (blockIdx.x == 0) {
+    const int i = threadIdx.x;
+    if (i < k) col[i] = h1[i] + h2[i];
+    if (i == 0) hn[0] = col[k] = norm;
+  }
+  const float2 g = df_from_double(1.0 / norm);
+  const size_t stride = (size_t)gridDim.x * blockDim.x;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += stride) {
+    const float2 a = w[i];                          // double-float product, renormalised
+    const float p = __fmul_rn(a.x, g.x);
+    float e = fmaf(a.x, g.x, -p);
+    e = fmaf(a.x, g.y, e);
+    e = fmaf(a.y, g.x, e);
+    const float hi = __fadd_rn(p, e);
+    const float2 r = make_float2(hi, __fsub_rn(e, __fsub_rn(hi, p)));
+    v[i] = r;
+    if constexpr (sizeof(TO) == 4) out[i] = __fadd_rn(r.x, r.y);
+    else out[i] = df_to_double(r);
   }
 }
 
@@ -609,8 +624,8 @@ int gs_blocks(size_t N) {
 }
 
 template <int K, int MODE, typename TW>
-cudaError_t launch_sweep_k(const float2* V, size_t ldv, const TW* w, const double* h, float2* wdf, size_t N,
-                           double* partial, int* nblk_out, cudaStream_t s) {
+cudaError_t launch_sweep_k(const float2* V, size_t ldv, const TW* w, const double* hpart, double* h, float2* wdf,
+                           size_t N, double* partial, int* nblk_out, cudaStream_t s) {
   using Sh = SweepShape<K>;
   auto kern = k_gs_sweep<K, MODE, TW>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem);
@@ -618,16 +633,14 @@ cudaError_t launch_sweep_k(const float2* V, size_t ldv, const TW* w, const doubl
   const size_t nchunk = (N + Sh::E - 1) / Sh::E;
   const int nblk = (int)(nchunk < 1 ? 1 : (nchunk > 152 ? 152 : nchunk));
   *nblk_out = nblk;
-  SBM_PDL(kern, nblk, kSweepThreads, Sh::smem, s, V, ldv, w, h, wdf, N, partial);
+  SBM_PDL(kern, nblk, kSweepThreads, Sh::smem, s, V, ldv, w, hpart, h, wdf, N, partial);
   return cudaSuccess;
 }
 
-// One staged sweep over nv basis vectors and the reduction of its per-block partial sums into out
-// (nv values for MODE 0 and 1, the norm for MODE 2).
+// One staged sweep over nv basis vectors (k_gs_sweep); nblk: its blocks.
 template <int MODE, typename TW>
-cudaError_t launch_sweep(const float2* V, size_t ldv, int nv, const TW* w, const double* h, float2* wdf, size_t N,
-                         double* partial, double* out, cudaStream_t s, const double* h1 = nullptr,
-                         double* col = nullptr) {
+cudaError_t launch_sweep(const float2* V, size_t ldv, int nv, const TW* w, const double* hpart, double* h, float2* wdf,
+                         size_t N, double* partial, int* nblk_out, cudaStream_t s) {
   if (nv < 1 || nv > kMaxVec) return cudaErrorInvalidValue;
   const size_t padded = N + (N & 1);
   if (ldv % 2 != 0 || ldv < padded || reinterpret_cast<uintptr_t>(V) % 16 != 0 ||
@@ -637,7 +650,7 @@ cudaError_t launch_sweep(const float2* V, size_t ldv, int nv, const TW* w, const
   cudaError_t e = cudaSuccess;
   switch (nv) {
 #define SBM_SW_CASE(K) \
-  case K: e = launch_sweep_k<K, MODE, TW>(V, ldv, w, h, wdf, N, partial, &nblk, s); break;
+  case K: e = launch_sweep_k<K, MODE, TW>(V, ldv, w, hpart, h, wdf, N, partial, &nblk, s); break;
     SBM_SW_CASE(1) SBM_SW_CASE(2) SBM_SW_CASE(3) SBM_SW_CASE(4) SBM_SW_CASE(5) SBM_SW_CASE(6)
     SBM_SW_CASE(7) SBM_SW_CASE(8) SBM_SW_CASE(9) SBM_SW_CASE(10) SBM_SW_CASE(11) SBM_SW_CASE(12)
     SBM_SW_CASE(13) SBM_SW_CASE(14) SBM_SW_CASE(15) SBM_SW_CASE(16) SBM_SW_CASE(17) SBM_SW_CASE(18)
@@ -647,36 +660,48 @@ cudaError_t launch_sweep(const float2* V, size_t ldv, int nv, const TW* w, const
 #undef SBM_SW_CASE
   }
   if (e != cudaSuccess) return e;
-  if (MODE == 2 && col) {                            // |w| and the Hessenberg column in one launch
-    if (nv + 1 > 64) return cudaErrorInvalidValue;
-    SBM_PDL(k_reduce_norm_column, 1, 64, 0, s, partial, nblk, out, h1, h, nv, col);
-  } else {
-    const int nout = MODE == 2 ? 1 : nv;
-    SBM_PDL(k_reduce_partials, 1, 32 * nout, 0, s, partial, nblk, nout, out, MODE == 2 ? 1 : 0);
-  }
-  count_launches(2);
+  if (nblk_out) *nblk_out = nblk;
+  count_launches();
   return cudaGetLastError();
 }
 
 cudaError_t launch_gs_dot(const float2* V, size_t ldv, int nv, const double* w, float2* wdf, size_t N,
-                          double* partial, double* out, cudaStream_t s) {
-  return launch_sweep<0, double>(V, ldv, nv, w, nullptr, wdf, N, partial, out, s);
+                          double* partial, cudaStream_t s) {
+  return launch_sweep<0, double>(V, ldv, nv, w, nullptr, nullptr, wdf, N, partial, nullptr, s);
 }
 
 cudaError_t launch_gs_dot_df(const float2* V, size_t ldv, int nv, const float2* wdf, size_t N, double* partial,
-                             double* out, cudaStream_t s) {
-  return launch_sweep<0, float2>(V, ldv, nv, wdf, nullptr, const_cast<float2*>(wdf), N, partial, out, s);
+                             cudaStream_t s) {
+  return launch_sweep<0, float2>(V, ldv, nv, wdf, nullptr, nullptr, const_cast<float2*>(wdf), N, partial, nullptr, s);
 }
 
-cudaError_t launch_gs_axpy_dot(const float2* V, size_t ldv, int nv, const double* h, float2* wdf, size_t N,
-                               double* partial, double* out, cudaStream_t s) {
-  return launch_sweep<1, float2>(V, ldv, nv, wdf, h, wdf, N, partial, out, s);
+cudaError_t launch_gs_axpy_dot(const float2* V, size_t ldv, int nv, const double* hpart, double* h, float2* wdf,
+                               size_t N, double* partial, cudaStream_t s) {
+  return launch_sweep<1, float2>(V, ldv, nv, wdf, hpart, h, wdf, N, partial, nullptr, s);
 }
 
-cudaError_t launch_gs_axpy_norm(const float2* V, size_t ldv, int nv, const double* h, float2* wdf, size_t N,
-                                double* partial, double* out, cudaStream_t s, const double* h1, double* col) {
-  return launch_sweep<2, float2>(V, ldv, nv, wdf, h, wdf, N, partial, out, s, h1, col);
+cudaError_t launch_gs_axpy_norm(const float2* V, size_t ldv, int nv, const double* hpart, double* h, float2* wdf,
+                                size_t N, double* partial, int* nblk, cudaStream_t s) {
+  return launch_sweep<2, float2>(V, ldv, nv, wdf, hpart, h, wdf, N, partial, nblk, s);
 }
+
+cudaError_t launch_gs_norm(const double* partial, int nblk, double* hn, cudaStream_t s) {
+  SBM_PDL(k_reduce_partials, 1, 32, 0, s, partial, nblk, 1, hn, 1);
+  count_launches();
+  return cudaGetLastError();
+}
+
+template <typename TO>
+cudaError_t launch_gs_scale_norm(const float2* w, const double* partial, int nblk, double* hn, const double* h1,
+                                 const double* h2, int k, double* col, float2* v, TO* out, size_t N, cudaStream_t s) {
+  SBM_PDL((k_gs_scale_norm<TO>), grid_for(N), 256, 0, s, w, partial, nblk, hn, h1, h2, k, col, v, out, N);
+  count_launches();
+  return cudaGetLastError();
+}
+template cudaError_t launch_gs_scale_norm<float>(const float2*, const double*, int, double*, const double*,
+                                                 const double*, int, double*, float2*, float*, size_t, cudaStream_t);
+template cudaError_t launch_gs_scale_norm<double>(const float2*, const double*, int, double*, const double*,
+                                                  const double*, int, double*, float2*, double*, size_t, cudaStream_t);
 
 int sweep_fault_take() {
   int f = 0;
@@ -688,20 +713,14 @@ int sweep_fault_take() {
   return f;
 }
 
-template <typename TW, typename TO>
-cudaError_t launch_gs_scale(const TW* w, const double* sc, float2* v, TO* out, size_t N, cudaStream_t s) {
-  SBM_PDL((k_gs_scale<TW, TO>), grid_for(N), 256, 0, s, w, sc, v, out, N);
+template <typename TO>
+cudaError_t launch_gs_scale(const double* w, const double* sc, float2* v, TO* out, size_t N, cudaStream_t s) {
+  SBM_PDL((k_gs_scale<TO>), grid_for(N), 256, 0, s, w, sc, v, out, N);
   count_launches();
   return cudaGetLastError();
 }
-template cudaError_t launch_gs_scale<double, float>(const double*, const double*, float2*, float*, size_t,
-                                                    cudaStream_t);
-template cudaError_t launch_gs_scale<double, double>(const double*, const double*, float2*, double*, size_t,
-                                                     cudaStream_t);
-template cudaError_t launch_gs_scale<float2, float>(const float2*, const double*, float2*, float*, size_t,
-                                                    cudaStream_t);
-template cudaError_t launch_gs_scale<float2, double>(const float2*, const double*, float2*, double*, size_t,
-                                                     cudaStream_t);
+template cudaError_t launch_gs_scale<float>(const double*, const double*, float2*, float*, size_t, cudaStream_t);
+template cudaError_t launch_gs_scale<double>(const double*, const double*, float2*, double*, size_t, cudaStream_t);
 
 template <typename TO>
 cudaError_t launch_df_to(const float2* v, TO* y, size_t N, cudaStream_t s) {

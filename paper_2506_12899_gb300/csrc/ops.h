@@ -336,28 +336,33 @@ cudaError_t launch_cast(const TI* x, TO* y, size_t N, cudaStream_t s);
 // c = a + b (k <= 32 entries), c[k] = hn at index k
 // Gram-Schmidt on a double-float basis V (pairs hi, lo of FP32 per entry, Dekker 1971), with w
 // carried between the sweeps as double-float in wdf:
-//   gs_dot:        wdf = w (FP64 in), out = V^T w
-//   gs_axpy_dot:   wdf -= V h, out = V^T wdf
-//   gs_axpy_norm:  wdf -= V h, out = |wdf|
-//   gs_scale:      v = w / s[0] (w FP64 or double-float), and out = v rounded to TO if non-null
-// The first four stream V and w through shared memory with bulk asynchronous copies: V, w and
+//   gs_dot:        wdf = w (FP64 in), partial sums of V^T w
+//   gs_axpy_dot:   wdf -= V h, partial sums of V^T wdf
+//   gs_axpy_norm:  wdf -= V h, partial sums of |wdf|^2
+// These stream V and w through shared memory with bulk asynchronous copies: V, w and
 // wdf must be 16-byte aligned, ldv even and >= N rounded up to even, and w / wdf hold that many
 // entries (cudaErrorInvalidValue otherwise).  A copy that does not complete in bounded time sets
 // a flag that sweep_fault_take() returns (1) and clears; -1 if the flag cannot be read.
 cudaError_t launch_gs_dot(const float2* V, size_t ldv, int nv, const double* w, float2* wdf, size_t N,
-                          double* partial, double* out, cudaStream_t s);
-// gs_dot with w already double-float (wdf, read only)
+                          double* partial, cudaStream_t s);
 cudaError_t launch_gs_dot_df(const float2* V, size_t ldv, int nv, const float2* wdf, size_t N, double* partial,
-                             double* out, cudaStream_t s);
-cudaError_t launch_gs_axpy_dot(const float2* V, size_t ldv, int nv, const double* h, float2* wdf, size_t N,
-                               double* partial, double* out, cudaStream_t s);
-// With col: also col[i] = h1[i] + h[i] (i < nv) and col[nv] = |wdf| (the Hessenberg column), in
-// the same reduction launch.
-cudaError_t launch_gs_axpy_norm(const float2* V, size_t ldv, int nv, const double* h, float2* wdf, size_t N,
-                                double* partial, double* out, cudaStream_t s, const double* h1 = nullptr,
-                                double* col = nullptr);
-template <typename TW, typename TO>
-cudaError_t launch_gs_scale(const TW* w, const double* sc, float2* v, TO* out, size_t N, cudaStream_t s);
+                             cudaStream_t s);
+// The update sweeps take h as the partial sums hpart of the sweep before and write it out (nv values); hpart
+// and partial are different buffers.  *nblk: the blocks of the norm sweep.
+cudaError_t launch_gs_axpy_dot(const float2* V, size_t ldv, int nv, const double* hpart, double* h, float2* wdf,
+                               size_t N, double* partial, cudaStream_t s);
+cudaError_t launch_gs_axpy_norm(const float2* V, size_t ldv, int nv, const double* hpart, double* h, float2* wdf,
+                                size_t N, double* partial, int* nblk, cudaStream_t s);
+// hn = |w| from the norm sweep's partial sums.
+cudaError_t launch_gs_norm(const double* partial, int nblk, double* hn, cudaStream_t s);
+// The same together with v = w / |w| (double-float, and rounded to TO in out) and the Hessenberg column
+// col[i] = h1[i] + h2[i] (i < k), col[k] = |w|.
+template <typename TO>
+cudaError_t launch_gs_scale_norm(const float2* w, const double* partial, int nblk, double* hn, const double* h1,
+                                 const double* h2, int k, double* col, float2* v, TO* out, size_t N, cudaStream_t s);
+// v = w / sc[0] as double-float and (out non-null) rounded to TO.
+template <typename TO>
+cudaError_t launch_gs_scale(const double* w, const double* sc, float2* v, TO* out, size_t N, cudaStream_t s);
 template <typename TO>
 cudaError_t launch_df_to(const float2* v, TO* y, size_t N, cudaStream_t s);
 cudaError_t launch_hess_column(const double* h1, const double* h2, const double* hn, int k, double* col,
