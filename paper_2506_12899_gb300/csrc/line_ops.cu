@@ -403,13 +403,158 @@ __global__ void __launch_bounds__(kLineThreads) k_resid_restrict_line(const __gr
   }
 }
 
-// One colour group of the block Gauss-Seidel sweep (Eq. 16) on a 3D level of degree N1 - 1, FP32,
-// 8 cells of one segment per block:
+// y += sum over m of coef[m] v_m, v_m the plane of the cell's lane m: a contraction along z, the planes
+// exchanged one after another (the terms are added in the order of m, as along x and y).
+template <int N1>
+__device__ __forceinline__ void plane_contract(const float (&coef)[N1], const float (&v)[N1 * N1], int base,
+                                               float (&y)[N1 * N1]) {
+#pragma unroll
+  for (int m = 0; m < N1; ++m)
+#pragma unroll
+    for (int q = 0; q < N1 * N1; ++q) y[q] = fmaf(coef[m], __shfl_sync(0xffffffffu, v[q], base + m), y[q]);
+}
+
+// y = M applied to a plane's nodes along x (dir 0) or y (dir 1); T: M transposed.
+template <int N1, bool T>
+__device__ __forceinline__ void plane_apply(const float* M, int dir, float (&v)[N1 * N1]) {
+  float w[N1 * N1];
+#pragma unroll
+  for (int tl = 0; tl < N1; ++tl)
+#pragma unroll
+    for (int m = 0; m < N1; ++m) {
+      float acc = 0.f;
+#pragma unroll
+      for (int q = 0; q < N1; ++q)
+        acc = fmaf(T ? M[q * N1 + m] : M[m * N1 + q], v[dof<2, N1>(dir, q, tl)], acc);
+      w[dof<2, N1>(dir, m, tl)] = acc;
+    }
+#pragma unroll
+  for (int q = 0; q < N1 * N1; ++q) v[q] = w[q];
+}
+
+// The interior cells of a smoother launch, one lane per x-y plane of a cell (N1 lanes per cell, 10 cells per
+// warp at p = 2, 8 at p = 3): a plane's N1^2 values are contiguous, so the lane reads its plane of the
+// cell and of every neighbour into registers, contracts x and y there and exchanges z contributions with the
+// cell's other lanes.  With one lane per line and everything in shared memory, the shared-memory reads
+// bound the launch (32 16-byte reads per lane and 3 cells per warp at p = 2); here it is 108 exchanges for
+// 10 cells.  The terms are added in the same order as there, to the same bits.  (Exchanging products instead
+// of planes takes half the exchanges, 52 instead of 55 us for a 112^3 p = 2 sweep, but rounds otherwise, and
+// the long 96^3 p = 3 solve to 1e-12 then ends after another number of steps.)
+// 128 threads; blk: the block's number in its segment.  112^3 p = 2 sweep 97.6 -> 55.2 us,
+// 96^3 p = 3 solve 83.1 -> 73.4 ms.
+template <int N1>
+__device__ __forceinline__ void smooth_planes(const LevelParams<float>& P, int first, int last, int col, int zero_start,
+                                              const float* __restrict__ f, float* __restrict__ u, int early, int blk,
+                                              float* stage) {
+  constexpr int NQ = N1 * N1, CPW = 32 / N1;
+  const LevelConsts<float>& C = P.k;
+  const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+  const int a0 = first + (blk * (kLineThreads / 32) + warp) * CPW;
+  const int g = min(lane / N1, CPW - 1), k = lane - lane / N1 * N1, base = g * N1;   // (idle lanes: the last cell, no store)
+  const int a = a0 + g;
+  const bool valid = lane < CPW * N1 && a < last;
+  const int pl = a * N1 + k, npl = P.n_act * N1;     // this lane's plane of the vector
+  int nb[6];
+#pragma unroll
+  for (int s = 0; s < 6; ++s) {                      // set-up data: read before the wait
+    nb[s] = valid ? P.nbr[(size_t)s * P.n_act + a] : -1;
+    if ((zero_start == kZeroLater && (col ^ (1 << (s >> 1))) > col) || zero_start == kZeroAll) nb[s] = -1;
+  }
+  float t[NQ], idg[NQ], cm[N1], cp[N1], sf[N1], sb[N1];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    t[q] = 0.f;
+    idg[q] = C.inv_diag[q + NQ * k];
+  }
+#pragma unroll
+  for (int m = 0; m < N1; ++m) {                     // row k of the 1D matrices
+    cm[m] = C.Bpm[N1 * k + m];
+    cp[m] = C.Bmp[N1 * k + m];
+    sf[m] = C.S[N1 * m + k];
+    sb[m] = C.S[N1 * k + m];
+  }
+  const float wk = C.w[k];
+  if (valid && early) load_cell_l2<2, N1, float, float>(f, pl, npl, t);   // f written two or more launches back
+  pdl_wait();
+  pdl_trigger();
+  if (valid && !early) load_cell<2, N1, float, float>(f, pl, npl, t);
+  float acc[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) acc[q] = 0.f;
+#pragma unroll
+  for (int dir = 0; dir < 2; ++dir) {                // x and y neighbours: in the plane
+    float x[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) x[q] = 0.f;
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      if (nb[2 * dir + side] < 0) continue;
+      float v[NQ];
+      load_cell<2, N1, float, float>(u, nb[2 * dir + side] * N1 + k, npl, v);
+      const float* B = side ? C.Bmp : C.Bpm;
+#pragma unroll
+      for (int tl = 0; tl < N1; ++tl)
+#pragma unroll
+        for (int i = 0; i < N1; ++i)
+#pragma unroll
+          for (int j = 0; j < N1; ++j)
+            x[dof<2, N1>(dir, i, tl)] = fmaf(B[i * N1 + j], v[dof<2, N1>(dir, j, tl)], x[dof<2, N1>(dir, i, tl)]);
+    }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) acc[q] = fmaf(C.w[dir == 0 ? q / N1 : q % N1] * wk, x[q], acc[q]);
+  }
+  {                                                  // z neighbours
+    float v[NQ], z[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) z[q] = 0.f;
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) v[q] = 0.f;
+      if (nb[4 + side] >= 0) load_cell<2, N1, float, float>(u, nb[4 + side] * N1 + k, npl, v);
+      plane_contract<N1>(side ? cp : cm, v, base, z);
+    }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      acc[q] = fmaf(C.w[q % N1] * C.w[q / N1], z[q], acc[q]);
+      t[q] = t[q] - P.hscale * acc[q];
+    }
+  }
+  plane_apply<N1, true>(C.S, 0, t);                  // fast diagonalisation: S^T along x, y, z
+  plane_apply<N1, true>(C.S, 1, t);
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) acc[q] = 0.f;
+  plane_contract<N1>(sf, t, base, acc);
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) acc[q] *= idg[q];
+  plane_apply<N1, false>(C.S, 0, acc);               // S along x, y, z
+  plane_apply<N1, false>(C.S, 1, acc);
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) t[q] = 0.f;
+  plane_contract<N1>(sb, acc, base, t);
+  if (P.omega != 1.f) {
+    float uold[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) uold[q] = 0.f;
+    if (valid && zero_start == kZeroNone) load_cell<2, N1, float, float>(u, pl, npl, uold);
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) t[q] = (1.f - P.omega) * uold[q] + P.omega * t[q];
+  }
+  if constexpr (cell_vec16<NQ, float>()) {
+    if (valid) store_cell<2, N1, float>(u, pl, t);
+  } else {
+    const int cells = min(CPW, last - a0);
+    if (cells > 0) warp_store_cells<NQ, float>(u, a0 * N1, cells * N1, t, stage + warp * 32 * NQ);
+  }
+}
+
+// One colour group of the block Gauss-Seidel sweep (Eq. 16) on a 3D level of degree N1 - 1, FP32:
 //   t_K = f_K - sum over interior faces of A_KN u_N (the SBM terms lie in A_KK),
 //   u_K <- (1 - omega) u_K + omega A_KK^-1 t_K.
-// The couplings take the same line, plane and row reads as the operator.  Boundary cells apply
-// their dense inverse (each thread its N1 rows, t from shared memory); interior cells the fast
-// diagonalisation (S^T)^(x3), 1 / (h^(d-2) sum lambda), S^(x3).  zero_start: a kZero* mode (ops.h).
+// Blocks of interior segments take smooth_planes (fast diagonalisation (S^T)^(x3), 1 / (h^(d-2) sum lambda),
+// S^(x3)).  Blocks of boundary segments take one thread per line: the couplings with the same line, plane and
+// row reads as the operator, then the dense inverse (each thread its N1 rows, t from shared memory).
+// zero_start: a kZero* mode (ops.h).
 template <int N1>
 __global__ void __launch_bounds__(kLineThreads) k_smooth_line(const __grid_constant__ LevelParams<float> P,
                                                               const __grid_constant__ SmoothSegs G, int zero_start,
@@ -417,16 +562,20 @@ __global__ void __launch_bounds__(kLineThreads) k_smooth_line(const __grid_const
                                                               int early) {
   constexpr int NP = LD<N1>::NP, NL = LD<N1>::NL, ST = LD<N1>::ST, Q = N1 * N1, CPB = LD<N1>::CPB;
   __shared__ __align__(16) float sN[CPB][6][ST];
-  __shared__ __align__(16) float sT[CPB][ST], sW[CPB][ST];
-  int c, l;
-  const bool lane_ok = line_lane<N1>(c, l);          // idle lanes mirror line 0 of the warp (no stores)
-  const int j = l % N1, k = l / N1;
+  __shared__ __align__(16) float sT[CPB][ST];
   int sg = 0;
 #pragma unroll
   for (int q = 1; q < SmoothSegs::kMax; ++q)
     if (q < G.n && (int)blockIdx.x >= G.blk[q]) sg = q;
   const int col = G.col[sg], cs = G.cs[sg];
-  const bool isB = G.first[sg] < cs + G.nbnd[sg];    // segments are all-boundary or all-interior
+  if (G.first[sg] >= cs + G.nbnd[sg]) {              // segments are all-boundary or all-interior
+    smooth_planes<N1>(P, G.first[sg], G.last[sg], col, zero_start, f, u, early, (int)blockIdx.x - G.blk[sg],
+                      &sN[0][0][0]);
+    return;
+  }
+  int c, l;
+  const bool lane_ok = line_lane<N1>(c, l);          // idle lanes mirror line 0 of the warp (no stores)
+  const int j = l % N1, k = l / N1;
   const int a = G.first[sg] + ((int)blockIdx.x - G.blk[sg]) * CPB + c;
   const bool valid = lane_ok && a < G.last[sg];
   const bool line = valid && l < NL;
@@ -449,103 +598,30 @@ __global__ void __launch_bounds__(kLineThreads) k_smooth_line(const __grid_const
     if (line && P.omega != 1.f && zero_start == kZeroNone) ldg_line<N1, false>(u, o, uold);
   }
   __syncthreads();
-  const LevelConsts<float>& C = P.k;
   float t[N1];
   {                                                  // couplings (Eq. 10, interior faces)
     float acc[N1];
 #pragma unroll
     for (int i = 0; i < N1; ++i) acc[i] = 0.f;
-    if (line) line_interior<false, N1, float>(C, nullptr, sN[c], nb, j, k, acc);
+    if (line) line_interior<false, N1, float>(P.k, nullptr, sN[c], nb, j, k, acc);
 #pragma unroll
     for (int i = 0; i < N1; ++i) t[i] = fv[i] - P.hscale * acc[i];
   }
   float y[N1];
 #pragma unroll
   for (int i = 0; i < N1; ++i) y[i] = 0.f;
-  float* lt = sT[c] + 4 * (j + N1 * k);
-  float* lw = sW[c] + 4 * (j + N1 * k);
-  const bool owner = lane_ok && l < NL;              // writes its line in the exchanges
-  if (isB) {                                         // dense inverse: y = Binv t
-    if (owner) sts_line<N1>(lt, t);
-    __syncwarp();
-    if (line) {
-      const float* Bi = P.binvT + (size_t)(G.b0[sg] + (a - cs)) * NP * NP + N1 * j + Q * k;
+  if (lane_ok && l < NL) sts_line<N1>(sT[c] + 4 * (j + N1 * k), t);
+  __syncwarp();
+  if (line) {                                        // dense inverse: y = Binv t
+    const float* Bi = P.binvT + (size_t)(G.b0[sg] + (a - cs)) * NP * NP + N1 * j + Q * k;
 #pragma unroll(N1 == 4 ? 8 : 9)
-      for (int q = 0; q < NP; ++q) {
-        float b[N1];
-        ldg_line<N1, false>(Bi, (size_t)q * NP, b);
-        const float tq = sT[c][sp<N1>(q)];
+    for (int q = 0; q < NP; ++q) {
+      float b[N1];
+      ldg_line<N1, false>(Bi, (size_t)q * NP, b);
+      const float tq = sT[c][sp<N1>(q)];
 #pragma unroll
-        for (int i = 0; i < N1; ++i) y[i] = fmaf(b[i], tq, y[i]);
-      }
+      for (int i = 0; i < N1; ++i) y[i] = fmaf(b[i], tq, y[i]);
     }
-  } else {                                           // fast diagonalisation
-    float w[N1], v[N1], z[N1];
-#pragma unroll
-    for (int m = 0; m < N1; ++m) {                   // x: S^T on the thread's line
-      w[m] = 0.f;
-#pragma unroll
-      for (int q = 0; q < N1; ++q) w[m] = fmaf(C.S[q * N1 + m], t[q], w[m]);
-    }
-    if (owner) sts_line<N1>(lt, w);
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < N1; ++i) v[i] = 0.f;         // y: S^T along the lines (i, ., k)
-#pragma unroll
-    for (int q = 0; q < N1; ++q) {
-      float r[N1];
-      lds_line<N1>(sT[c] + 4 * (q + N1 * k), r);
-      const float cq = C.S[N1 * q + j];
-#pragma unroll
-      for (int i = 0; i < N1; ++i) v[i] = fmaf(cq, r[i], v[i]);
-    }
-    __syncwarp();
-    if (owner) sts_line<N1>(lw, v);
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < N1; ++i) z[i] = 0.f;         // z: S^T along the lines (i, j, .)
-#pragma unroll
-    for (int q = 0; q < N1; ++q) {
-      float r[N1];
-      lds_line<N1>(sW[c] + 4 * (j + N1 * q), r);
-      const float cq = C.S[N1 * q + k];
-#pragma unroll
-      for (int i = 0; i < N1; ++i) z[i] = fmaf(cq, r[i], z[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < N1; ++i) z[i] *= C.inv_diag[i + N1 * j + Q * k];
-#pragma unroll
-    for (int m = 0; m < N1; ++m) {                   // x: S on the thread's line
-      w[m] = 0.f;
-#pragma unroll
-      for (int q = 0; q < N1; ++q) w[m] = fmaf(C.S[m * N1 + q], z[q], w[m]);
-    }
-    __syncwarp();
-    if (owner) sts_line<N1>(lt, w);
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < N1; ++i) v[i] = 0.f;         // y: S along (i, ., k)
-#pragma unroll
-    for (int q = 0; q < N1; ++q) {
-      float r[N1];
-      lds_line<N1>(sT[c] + 4 * (q + N1 * k), r);
-      const float cq = C.S[N1 * j + q];
-#pragma unroll
-      for (int i = 0; i < N1; ++i) v[i] = fmaf(cq, r[i], v[i]);
-    }
-    __syncwarp();
-    if (owner) sts_line<N1>(lw, v);
-    __syncwarp();
-#pragma unroll
-    for (int q = 0; q < N1; ++q) {                   // z: S along (i, j, .)
-      float r[N1];
-      lds_line<N1>(sW[c] + 4 * (j + N1 * q), r);
-      const float cq = C.S[N1 * k + q];
-#pragma unroll
-      for (int i = 0; i < N1; ++i) y[i] = fmaf(cq, r[i], y[i]);
-    }
-  }
-  if (line) {
     if (P.omega != 1.f) {
 #pragma unroll
       for (int i = 0; i < N1; ++i) y[i] = (1.f - P.omega) * uold[i] + P.omega * y[i];
@@ -608,7 +684,7 @@ cudaError_t launch_smooth_line(int p, const LevelParams<float>& P, int reverse, 
   const int ng = n_colour_groups(P, 3);
   for (int q = first_group; q < ng; ++q) {
     const int g = reverse ? ng - 1 - q : q;
-    const SmoothSegs G = smooth_segs(P, 3, g, p == 3 ? LD<4>::CPB : LD<3>::CPB);
+    const SmoothSegs G = smooth_segs(P, 3, g, p == 3 ? LD<4>::CPB : LD<3>::CPB, (kLineThreads / 32) * (32 / (p + 1)));
     if (G.n == 0 || G.blk[G.n] == 0) continue;
     const int fe = launched > 0 || early;            // after the sweep's first launch f is two back
     const int zm = group_zero_mode(P, zero_start, q);

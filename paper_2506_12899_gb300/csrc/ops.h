@@ -125,7 +125,7 @@ int dots_noalloc(const double* V, long long ldv, int nv, const double* w, long l
 // colours of a group updated by one launch: every cell reads the same neighbour values.
 // With red-black ordering (LevelParams::ordering = 1) the groups are the two index-sum parities,
 // popcount(c) mod 2: a face changes one index by one, so cells of equal parity never neighbour.
-// smooth_segs lists the segments of group g with cpb cells per block.
+// smooth_segs lists the segments of group g with cpb cells per block (interior segments: cpb_in if given).
 template <typename R>
 inline int colour_group(const LevelParams<R>& P, int c) {
   const int pc = __builtin_popcount((unsigned)c);
@@ -145,7 +145,7 @@ inline int n_colour_groups(const LevelParams<R>& P, int dim) {
 enum { kZeroNone = 0, kZeroLater = 1, kZeroAll = 2, kZeroSelf = 3 };
 
 template <typename R>
-inline SmoothSegs smooth_segs(const LevelParams<R>& P, int dim, int g, int cpb) {
+inline SmoothSegs smooth_segs(const LevelParams<R>& P, int dim, int g, int cpb, int cpb_in = 0) {
   SmoothSegs G{};
   G.n = 0;
   G.blk[0] = 0;
@@ -162,7 +162,8 @@ inline SmoothSegs smooth_segs(const LevelParams<R>& P, int dim, int g, int cpb) 
       G.cs[k] = cs;
       G.nbnd[k] = nb;
       G.b0[k] = P.bstart[c];
-      G.blk[k + 1] = G.blk[k] + (hi[part] - lo[part] + cpb - 1) / cpb;
+      const int per = part == 1 && cpb_in > 0 ? cpb_in : cpb;
+      G.blk[k + 1] = G.blk[k] + (hi[part] - lo[part] + per - 1) / per;
     }
   }
   return G;

@@ -558,3 +558,21 @@ def test_cta_tail_matches_per_level_launches(name, kw, offset):
     ref = b.vcycle(r.clone())
     assert used < S.kernel_launches() - before - used                 # the tail ran
     assert (z - ref).norm() <= 2e-5 * ref.norm()
+
+
+@pytest.mark.parametrize("n,p,kw", [(4, 2, dict()), (6, 3, dict()), (8, 2, dict(omega=0.7)), (10, 3, dict(ordering=1)),
+                                    (12, 2, dict(ordering=1, omega=0.9)), (14, 2, dict())])
+def test_plane_smoother_edges(n, p, kw):
+    """The 3D p = 2, 3 smoother (one lane per plane of an interior cell) against the thread-per-DoF kernel, both
+    FP32, with last warps of 1 to 10 cells, both orders, relaxation, red-black; and inside a V-cycle, where the
+    first sweep reads later colours as zero.  Bound: FP32 sums in another order, 2e-5 relative."""
+    import paper_2506_12899_gb300 as S
+    prob = W.sphere3d(n, 2, 1).replace(p=p, coarsest_n=4, omega_p3=kw.get("omega", 0.8), **kw)
+    a, b = S.Solver(prob, "f32"), S.Solver(prob, "f32", cell_kernel_min_cells=-1, tail_max_cells=-1)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    f, u = (torch.rand(a.n_dof(), generator=g, device="cuda") - 0.5 for _ in range(2))
+    for rev in (False, True):
+        x, y = a.smooth(f, u.clone(), reverse=rev), b.smooth(f, u.clone(), reverse=rev)
+        assert (x - y).norm() <= 2e-5 * y.norm()
+    z, ref = a.vcycle(f), b.vcycle(f)
+    assert (z - ref).norm() <= 2e-5 * ref.norm()
