@@ -607,7 +607,7 @@ Context* build_context(const sbm_setup_desc& d, bool device) {
       L.P64.bnd_ld = L.P32.bnd_ld = (int)ld;
       if (d.cell_kernel_min_cells >= 0) L.P32.binvS = C->upload(to_f32(bs));
       if (d.cell_kernel_min_cells > 0) L.P64.binvS = C->upload(bs);
-      if (d.cell_kernel_min_cells >= 0 && L.H.p == 1) L.P32.aselfS = C->upload(to_f32(by_entry(L.H.aselfT)));
+      if (d.cell_kernel_min_cells >= 0 && L.H.p == 1 && L.H.dim == 2) L.P32.aselfS = C->upload(to_f32(by_entry(L.H.aselfT)));
     }
     if (&L == &C->lv.back()) {                     // Arnoldi operator in double-float
       std::vector<dfl> dh(L.H.dhat.size());
@@ -719,14 +719,14 @@ size_t build_tail_cta(Context& C, int top, TailCta<R>& T) {
   }
   auto fits = [&] { return tail_cta_fits(dim, pi, bytes + 2 * vec); };
   if (!fits()) return 0;
-  // the coarse inverse, then the boundary self blocks from the smallest level up, where they still fit
+  // the coarse inverse, then (2D) the boundary self blocks from the smallest level up, where they still fit
   size_t keep = bytes;
   T.cinv = take(n0 * n0 * 8);
   if (!fits()) {
     bytes = keep;
     T.cinv = 0;
   }
-  for (int l = 1; l <= top; ++l) {
+  for (int l = 1; l <= top && dim == 2; ++l) {
     keep = bytes;
     D[l].aself = take(C.lv[l].H.n_bnd * blk);
     if (fits()) continue;
@@ -749,8 +749,8 @@ size_t build_tail_cta(Context& C, int top, TailCta<R>& T) {
     R* M = reinterpret_cast<R*>(&image[D[l].mats]);
     const double hs = std::pow(H.h, dim - 2), wt = dim == 2 ? H.B.w[0] : H.B.w[0] * H.B.w[0];
     for (int q = 0; q < 4; ++q) {
-      M[q] = (R)(hs * wt * H.Bpm[q]);
-      M[4 + q] = (R)(hs * wt * H.Bmp[q]);
+      M[q] = dim == 2 ? (R)(hs * wt * H.Bpm[q]) : (R)H.Bpm[q];   // 3D: weighted in the kernel
+      M[4 + q] = dim == 2 ? (R)(hs * wt * H.Bmp[q]) : (R)H.Bmp[q];
     }
     for (int i = 0; i < np; ++i)
       for (int j = 0; j < np; ++j) {
@@ -792,7 +792,7 @@ size_t build_tail_cta(Context& C, int top, TailCta<R>& T) {
           const int a = Hc.children[(size_t)o * Hc.n_act + cc];
           ch[(size_t)cc * ncol + o] = a >= 0 ? (uint16_t)a : 0xffff;
         }
-      if (!D[l].aself) T.aselfT[l] = C.upload(std::vector<R>(H.aselfT.begin(), H.aselfT.end()));
+      if (!D[l].aself && dim == 2) T.aselfT[l] = C.upload(std::vector<R>(H.aselfT.begin(), H.aselfT.end()));
     }
     T.omega[l] = (R)H.omega;
   }
@@ -811,8 +811,8 @@ size_t build_tail_cta(Context& C, int top, TailCta<R>& T) {
   T.image_bytes = (unsigned)bytes;
   T.vec_bytes = (unsigned)vec;
   T.image = C.upload(image);
-  for (int o = 0; o < 2; ++o)
-    for (int q = 0; q < 4; ++q) T.Ph[o][q] = tparams<R>(C.lv[1]).Ph[o][q];
+  T.T = tparams<R>(C.lv[1]);
+  for (int l = 0; l <= top; ++l) T.P[l] = params<R>(C.lv[l]);
   return bytes + 2 * vec;
 }
 

@@ -227,9 +227,9 @@ __device__ __forceinline__ R h_weight(const TransferParams<R>& T, int o, int i, 
 // SM0: also the first colour group of the coarse level's first pre-smoothing sweep from zero (see
 // k_resid_restrict_p_cell), computed by lane 0 of each coarse cell's group.
 //
-// PRE (as in k_smooth_cell): the children's self blocks, instead of their surrogate-face terms, and with SM0 the
-// coarse cells' inverses are read before the dependency wait: V-cycle of the 64^3 p = 1 sphere 79.0 -> 77.2 us.
-// (Not at 2D p = 2, k_resid_restrict_p_cell: 81 registers of block made that V-cycle 1.8 us longer; nor after the
+// PRE (as in k_smooth_cell): with SM0 the coarse cells' inverses, and in 2D the children's self blocks instead
+// of their surrogate-face terms, are read before the dependency wait: V-cycle of the 512^2 p = 2 star 95.7 ->
+// 94.1 us.  (3D keeps the order of its operations, see k_vcycle_tail_cta.  Not at 2D p = 2, k_resid_restrict_p_cell: 81 registers of block made that V-cycle 1.8 us longer; nor after the
 // wait in the operator: 44 -> 46 us at 2048^2 p = 2.)
 template <int D, typename R, bool SM0, bool PRE>
 __global__ void __launch_bounds__(PRE ? 32 : kCellThreads) k_resid_restrict_h_cell(const __grid_constant__ LevelParams<R> P,
@@ -249,12 +249,12 @@ __global__ void __launch_bounds__(PRE ? 32 : kCellThreads) k_resid_restrict_h_ce
   const int a = cc < T.n_act_c ? T.children[(size_t)o * T.n_act_c + cc] : -1;
   int nb[2 * D];
   R fa[NP];
-  constexpr int NPRE = PRE ? NP * NP : 1, NPRC = PRE && SM0 ? NP * NP : 1;
+  constexpr int NPRE = PRE && D == 2 ? NP * NP : 1, NPRC = PRE && SM0 ? NP * NP : 1;
   R A[NPRE], B[NPRC];
   if (a >= 0) {
     load_nbr<D, R>(P, a, nb);
     if (early) load_cell_l2<D, 2, R, R>(f, a, P.n_act, fa);   // f written two or more launches back
-    if constexpr (PRE) load_block<NPRE>(P.aselfS, P.bnd_ld, boundary_index(P, a, 1 << D), A);
+    if constexpr (PRE && D == 2) load_block<NPRE>(P.aselfS, P.bnd_ld, boundary_index(P, a, 1 << D), A);
   }
   if constexpr (PRE && SM0)
     load_block<NPRC>(Pc.binvS, Pc.bnd_ld, o == 0 && cc < T.n_act_c && cc < Pc.colour_nbnd[0] ? Pc.bstart[0] + cc : -1, B);
@@ -533,8 +533,11 @@ __device__ int g_tail_fault;
 //   - every phase's code appears once, in one loop over the levels down and up again, so the instructions
 //     of a phase are in the cache from its first use on;
 //   - a cell's neighbours, boundary index and parent are one 16-byte record; a missing neighbour is a
-//     zero cell, so no load waits for a branch; an interior cell applies a dense inverse like a
-//     boundary cell, so a warp of both takes one path;
+//     zero cell, so no load waits for a branch;
+//   - 2D: an interior cell applies a dense inverse like a boundary cell, so a warp of both takes one path,
+//     and boundary residuals use stored self blocks.  3D keeps the operations of the per-level kernels in
+//     their order, to the same bits: the long 3D p = 3 solves (96^3 to 1e-12) end after another number of
+//     steps when the rounding of their V-cycle changes;
 //   - vectors and blocks are laid out free of bank conflicts (TailCta).
 // What is left is bound by the shared-memory reads of the largest level's phases (the 64^2 level: 850 to
 // 1500 cycles a colour group, 4200 the restriction) and by each thread's chain on the smaller ones (500 to
@@ -564,8 +567,8 @@ __global__ void __launch_bounds__(kTailCtaThreads, 1) k_vcycle_tail_cta(const __
   R P0[4], P1[4];                                    // 1D transfer matrices of the two children
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    P0[q] = TP.Ph[0][q];
-    P1[q] = TP.Ph[1][q];
+    P0[q] = TP.T.Ph[0][q];
+    P1[q] = TP.T.Ph[1][q];
   }
   __syncthreads();                                   // the barrier is initialised before anyone polls it
   if (!__syncthreads_and(mbar_wait(&tbar, 0))) {     // record, let the copy land, copy by hand
@@ -598,7 +601,25 @@ __global__ void __launch_bounds__(kTailCtaThreads, 1) k_vcycle_tail_cta(const __
       store_np_vec<PW, R>(reinterpret_cast<R*>(tcta_smem + v + (unsigned)(w * (n + 1) + (int)a) * 16u), t);
     }
   };
-  // t -= the couplings to the neighbours of the record q (Eq. 10)
+  // 3D: c += the couplings to the neighbours of the record q, unscaled
+  auto couple3 = [&](const uint4& q, unsigned z, int n, const R(&b)[8], R wt, R(&c)[NP]) {
+    const unsigned w[3] = {q.x, q.y, q.z};
+#pragma unroll
+    for (int s = 0; s < 2 * D; ++s) {
+      R u[NP];
+      load(z, n, (s & 1) ? w[s >> 1] >> 16 : w[s >> 1] & 0xffffu, u);
+#pragma unroll
+      for (int tl = 0; tl < NP / 2; ++tl)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          // explicit: the compiler is free to fuse either product of a sum of two
+          R acc = fma(b[4 * (s & 1) + 2 * i], u[dof<D, 2>(s >> 1, 0, tl)], R(0));
+          acc = fma(b[4 * (s & 1) + 2 * i + 1], u[dof<D, 2>(s >> 1, 1, tl)], acc);
+          c[dof<D, 2>(s >> 1, i, tl)] += wt * acc;
+        }
+    }
+  };
+  // 2D: t -= the couplings to the neighbours of the record q (Eq. 10)
   auto couple = [&](const uint4& q, unsigned z, int n, const R(&b)[8], R(&t)[NP]) {
     const unsigned w[3] = {q.x, q.y, q.z};
 #pragma unroll
@@ -714,19 +735,29 @@ __global__ void __launch_bounds__(kTailCtaThreads, 1) k_vcycle_tail_cta(const __
         R e[NP], u[NP];
         load(zc, nc, code >> 3, e);
         load(z, n, a, u);
+        if constexpr (D == 3) {
 #pragma unroll
-        for (int dir = 0; dir < D; ++dir) {
-          const bool hi = (code >> dir) & 1u;
+          for (int i = 0; i < NP; ++i) {
+            R acc = 0;
 #pragma unroll
-          for (int tl = 0; tl < NP / 2; ++tl) {
-            const int i0 = dof<D, 2>(dir, 0, tl), i1 = dof<D, 2>(dir, 1, tl);
-            const R e0 = e[i0], e1 = e[i1];
-            e[i0] = (hi ? P1[0] : P0[0]) * e0 + (hi ? P1[1] : P0[1]) * e1;
-            e[i1] = (hi ? P1[2] : P0[2]) * e0 + (hi ? P1[3] : P0[3]) * e1;
+            for (int j = 0; j < NP; ++j) acc += h_weight<D, R>(TP.T, (int)(code & 7u), i, j) * e[j];
+            u[i] += acc;
           }
-        }
+        } else {
 #pragma unroll
-        for (int i = 0; i < NP; ++i) u[i] += e[i];
+          for (int dir = 0; dir < D; ++dir) {
+            const bool hi = (code >> dir) & 1u;
+#pragma unroll
+            for (int tl = 0; tl < NP / 2; ++tl) {
+              const int i0 = dof<D, 2>(dir, 0, tl), i1 = dof<D, 2>(dir, 1, tl);
+              const R e0 = e[i0], e1 = e[i1];
+              e[i0] = (hi ? P1[0] : P0[0]) * e0 + (hi ? P1[1] : P0[1]) * e1;
+              e[i1] = (hi ? P1[2] : P0[2]) * e0 + (hi ? P1[3] : P0[3]) * e1;
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < NP; ++i) u[i] += e[i];
+        }
         store(z, n, a, u);
       }
       __syncthreads();
@@ -745,11 +776,19 @@ __global__ void __launch_bounds__(kTailCtaThreads, 1) k_vcycle_tail_cta(const __
           const uint4 q = rec[a];
           R t[NP], y[NP];
           load(f, n, a, t);
-          couple(q, z, n, bc, t);
           const unsigned b = q.w & 0xffffu;
 #pragma unroll
           for (int i = 0; i < NP; ++i) y[i] = R(0);
-          block(b == 0xffffu ? M + 8 : reinterpret_cast<const R*>(tcta_smem + binv + b * BLK), t, R(1), y);
+          if constexpr (D == 3) {
+            const LevelParams<R>& LP = TP.P[l];
+            couple3(q, z, n, bc, LP.k.w[0] * LP.k.w[0], y);
+#pragma unroll
+            for (int i = 0; i < NP; ++i) t[i] -= LP.hscale * y[i];
+            block_solve_at<D, 2, R>(LP, b == 0xffffu ? nullptr : reinterpret_cast<const R*>(tcta_smem + binv + b * BLK), t, y);
+          } else {
+            couple(q, z, n, bc, t);
+            block(b == 0xffffu ? M + 8 : reinterpret_cast<const R*>(tcta_smem + binv + b * BLK), t, R(1), y);
+          }
           if (om != R(1)) {
             R uo[NP];
             load(z, n, a, uo);
@@ -781,6 +820,32 @@ __global__ void __launch_bounds__(kTailCtaThreads, 1) k_vcycle_tail_cta(const __
           R u[NP];
           load(z, n, a, u);
           load(f, n, a, r);
+          if constexpr (D == 3) {
+            const LevelParams<R>& LP = TP.P[l];
+            const unsigned w[3] = {q.x, q.y, q.z};
+            int nb[2 * D];
+#pragma unroll
+            for (int s = 0; s < 2 * D; ++s) {
+              const int m = (int)((s & 1) ? w[s >> 1] >> 16 : w[s >> 1] & 0xffffu);
+              nb[s] = m == n ? -1 : m;
+            }
+            R y[NP], out[NP];
+#pragma unroll
+            for (int i = 0; i < NP; ++i) y[i] = 0;
+            add_self<D, 2, R>(LP, nb, b == 0xffffu ? -1 : (int)b, u, y);
+            couple3(q, z, n, bc, LP.k.w[0] * LP.k.w[0], y);
+#pragma unroll
+            for (int i = 0; i < NP; ++i) r[i] = r[i] - LP.hscale * y[i];
+#pragma unroll
+            for (int j = 0; j < NP; ++j) {
+              R acc = 0;
+#pragma unroll
+              for (int i = 0; i < NP; ++i) acc += h_weight<D, R>(TP.T, o, i, j) * r[i];
+              out[j] = acc;
+            }
+#pragma unroll
+            for (int j = 0; j < NP; ++j) r[j] = out[j];
+          } else {
           if (aself) block(b == 0xffffu ? M + 8 + NP * NP : reinterpret_cast<const R*>(tcta_smem + aself + b * BLK), u, R(-1), r);
           else block(b == 0xffffu ? M + 8 + NP * NP : TP.aselfT[l] + b * (NP * NP), u, R(-1), r);
           couple(q, z, n, bc, r);
@@ -794,6 +859,7 @@ __global__ void __launch_bounds__(kTailCtaThreads, 1) k_vcycle_tail_cta(const __
               r[i0] = (hi ? P1[0] : P0[0]) * e0 + (hi ? P1[2] : P0[2]) * e1;
               r[i1] = (hi ? P1[1] : P0[1]) * e0 + (hi ? P1[3] : P0[3]) * e1;
             }
+          }
           }
         }
         // the sum over the children: at each exchange a lane keeps half of the values
@@ -937,7 +1003,7 @@ cudaError_t launch_resid_restrict_h_cell(int dim, const LevelParams<R>& P, const
   const bool sm0 = Pc != nullptr && zc != nullptr;
   const LevelParams<R>& Q = sm0 ? *Pc : P;
   constexpr bool kPre = sizeof(R) == 4;
-  const bool pre = kPre && bs == 32 && P.aselfS && (!sm0 || Q.binvS);
+  const bool pre = kPre && bs == 32 && (dim == 3 || P.aselfS) && (!sm0 || Q.binvS);
 #define SBM_RRHC(D)                                                                                               \
   {                                                                                                               \
     if (sm0 && pre) SBM_PDL((k_resid_restrict_h_cell<D, R, true, kPre>), g, bs, 0, s, P, T, u, f, rc, early, Q, zc); \

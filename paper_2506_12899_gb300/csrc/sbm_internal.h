@@ -209,7 +209,8 @@ struct TailCta {
   const void* image;
   const R* aselfT[kMaxTailCta];    // boundary self blocks in global memory, NP * NP each
   R omega[kMaxTailCta];
-  R Ph[2][4];
+  TransferParams<R> T;             // Ph: the 1D transfer matrices (p = 1, the same on every level)
+  LevelParams<R> P[kMaxTailCta];   // 3D: the level's 1D matrices
 };
 
 // Launch shape of the cluster tail of one precision: cluster size (CTAs), dynamic shared
