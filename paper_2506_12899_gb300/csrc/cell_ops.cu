@@ -539,10 +539,11 @@ __device__ int g_tail_fault;
 //     their order, to the same bits: the long 3D p = 3 solves (96^3 to 1e-12) end after another number of
 //     steps when the rounding of their V-cycle changes;
 //   - vectors and blocks are laid out free of bank conflicts (TailCta).
-// What is left is bound by the shared-memory reads of the largest level's phases (the 64^2 level: 850 to
+// What is left in 2D is bound by the shared-memory reads of the largest level's phases (the 64^2 level: 850 to
 // 1500 cycles a colour group, 4200 the restriction) and by each thread's chain on the smaller ones (500 to
-// 600 cycles).  A V-cycle of the 512^2 p = 2 star (tail: 64^2 .. 8^2) went 127 -> 107 us, one of a 64^3 p = 1
-// sphere (16^3 .. 4^3; its boundary self blocks stay in global memory) 153 -> 108 us.
+// 600 cycles): a V-cycle of the 512^2 p = 2 star (tail: 64^2 .. 8^2) went 127 -> 107 us. In 3D the restriction
+// of the largest level, with the surrogate-face terms of its boundary cells, is the longest phase: a V-cycle
+// of a 64^3 p = 1 sphere (16^3 .. 4^3) takes 89 us with this order of operations and 76 with the 2D form.
 template <int D, typename R>
 __global__ void __launch_bounds__(kTailCtaThreads, 1) k_vcycle_tail_cta(const __grid_constant__ TailCta<R> TP,
                                                                         const R* __restrict__ r_top,

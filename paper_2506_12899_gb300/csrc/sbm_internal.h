@@ -194,7 +194,7 @@ constexpr int kMaxTailCta = 6;
 constexpr int kTailMats = 136;     // coupling entries (8), interior inverse, interior block
 struct TailLevelDesc {
   int n_act;
-  unsigned z, f, binv, aself, mats, rec, ch;   // aself 0: the boundary self blocks stay in global memory
+  unsigned z, f, binv, aself, mats, rec, ch;   // aself 0: the boundary self blocks stay in global memory (3D: not used)
   // cell idx (0 <= idx < end2) of a colour group: idx + first0 below end0, + first1 below end1, + first2
   // below end2 (a group has up to three colours, each a range of cells)
   struct Group {
