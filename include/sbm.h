@@ -342,9 +342,15 @@ int sbm_mlp_set_params(void* mlp, const float* params_host);
 int sbm_mlp_get_params(const void* mlp, float* params_host);
 /* GEMM implementation of the MLP: 0 (default) the tcgen05 tensor-core kernels (128-row tiles, FP32
  * accumulators in tensor memory), 1 the warp-level mma.sync kernel.  Both compute the same
- * BF16 x BF16 -> FP32 products (summation order differs).  A tensor-core commit that does not arrive
- * within a bounded wait makes the next synchronising MLP call return SBM_ERR_CUDA. */
+ * BF16 x BF16 -> FP32 products (summation order differs).  Every wait of the tcgen05 kernels is
+ * bounded.  One that runs out sets a flag of this network: its outputs are zero (a correction of zero
+ * inside sbm_vcycle), and the next call that synchronises and uses the network (sbm_mlp_gradients,
+ * sbm_mlp_train, sbm_solve with the network attached) returns SBM_ERR_CUDA and clears the flag. */
 int sbm_mlp_gemm_backend(void* mlp, int backend);
+/* Polls after which a wait inside the one-launch kernel gives up: < 0 the default (2^22, also the
+ * largest), 0 at once (for tests of the failure path).  A context takes the value at its first
+ * solve after sbm_attach_mlp. */
+int sbm_mlp_wait_limit(void* mlp, int polls);
 /* Y_dev[rows][O] = MLP(X_dev[rows][F]) (device FP32 buffers; X is rounded to BF16). */
 int sbm_mlp_forward(void* mlp, const float* X_dev, int rows, float* Y_dev);
 /* Gradient of the mean squared error mean((MLP(X) - T)^2) over the rows x O entries, in the

@@ -67,8 +67,8 @@ struct DevLevel {
 // The MLP's GEMMs: tcgen05 (backend 0) or mma.sync (1).
 inline cudaError_t gemm_bf16(int backend, int M, int N, int K, int ta, int tb, const __nv_bfloat16* A, int lda,
                              const __nv_bfloat16* B, int ldb, const float* bias, int relu, float* Cf,
-                             __nv_bfloat16* Cb, int ldc, cudaStream_t s) {
-  return backend == 0 ? launch_gemm_tc(M, N, K, ta, tb, A, lda, B, ldb, bias, relu, Cf, Cb, ldc, s)
+                             __nv_bfloat16* Cb, int ldc, int* fault, cudaStream_t s) {
+  return backend == 0 ? launch_gemm_tc(M, N, K, ta, tb, A, lda, B, ldb, bias, relu, Cf, Cb, ldc, fault, s)
                       : launch_gemm_bf16(M, N, K, ta, tb, A, lda, B, ldb, bias, relu, Cf, Cb, ldc, s);
 }
 
@@ -85,6 +85,8 @@ struct Mlp {
   __nv_bfloat16* Wb = nullptr;       // the BF16 weight copies (MlpWeights)
   int adam_t = 0;
   int gemm = 0;                      // 0: tcgen05 tensor cores (tc_gemm.cu), 1: warp-level mma.sync
+  int* fault = nullptr;              // device flag: a tensor-core wait of this network ran out
+  unsigned spin = kAsyncSpin;        // polls of a wait in the one-launch kernel
   size_t cap = 0, count = 0;         // training set rows
   __nv_bfloat16* Xd = nullptr;       // [cap][Fpad]
   float* Td = nullptr;               // [cap][O]
@@ -152,6 +154,8 @@ struct Mlp {
     T.Op = Op;
     T.early = early;
     T.y_vec = reinterpret_cast<uintptr_t>(Yout) % 16 == 0;
+    T.spin = spin;
+    T.fault = fault;
     T.Xf = Xf;
     T.Xb = X;
     const MlpWeights M = weights();
@@ -204,9 +208,9 @@ struct Mlp {
   // Yout[rows][O] = MLP(X) with the BF16 weights, hidden activations into h1, h2 ([rows][H]).
   void forward(const __nv_bfloat16* X, int rows, float* Yout, __nv_bfloat16* h1, __nv_bfloat16* h2,
                cudaStream_t st) const {
-    CUDA_TRY(gemm_bf16(gemm, rows, H, Fpad, 0, 0, X, Fpad, W1b(), Hp, P + ob1, 1, nullptr, h1, H, st));
-    CUDA_TRY(gemm_bf16(gemm, rows, H, H, 0, 0, h1, H, W2b(), Hp, P + ob2, 1, nullptr, h2, H, st));
-    CUDA_TRY(gemm_bf16(gemm, rows, O, H, 0, 0, h2, H, W3b(), Op, P + ob3, 0, Yout, nullptr, O, st));
+    CUDA_TRY(gemm_bf16(gemm, rows, H, Fpad, 0, 0, X, Fpad, W1b(), Hp, P + ob1, 1, nullptr, h1, H, fault, st));
+    CUDA_TRY(gemm_bf16(gemm, rows, H, H, 0, 0, h1, H, W2b(), Hp, P + ob2, 1, nullptr, h2, H, fault, st));
+    CUDA_TRY(gemm_bf16(gemm, rows, O, H, 0, 0, h2, H, W3b(), Op, P + ob3, 0, Yout, nullptr, O, fault, st));
   }
   // G = gradient of the mean squared error over the rows of (X, T), X FP32 (Xf) or BF16 in the batch
   // buffer Xb (Xf null); loss_part receives partial sums of the squared errors.
@@ -238,6 +242,7 @@ struct Mlp {
     }
     if (!bias_part) bias_part = alloc<float>((size_t)kLossParts * (2 * Hp + Op));
     A.part = grad_part;
+    A.fault = fault;
     MlpTile t = tile(rows, Xf, Xf ? nullptr : Xb, nullptr, 0);
     t.T = T;
     t.inv_count = 1.0f / ((float)rows * O);
@@ -256,15 +261,15 @@ struct Mlp {
   // H1, H2); loss_part receives per-block partial sums of the squared errors.
   void backward(const __nv_bfloat16* X, const float* T, int rows) {
     CUDA_TRY(launch_mse_grad(rows, O, Y, T, dYf, dYb, 1.0f / ((float)rows * O), loss_part, 152, s));
-    CUDA_TRY(gemm_bf16(gemm, H, O, rows, 1, 0, H2, H, dYb, O, nullptr, 0, G + oW3, nullptr, O, s));
+    CUDA_TRY(gemm_bf16(gemm, H, O, rows, 1, 0, H2, H, dYb, O, nullptr, 0, G + oW3, nullptr, O, fault, s));
     CUDA_TRY(launch_colsum(rows, O, dYf, G + ob3, s));
-    CUDA_TRY(gemm_bf16(gemm, rows, H, O, 0, 1, dYb, O, W3b(), Op, nullptr, 0, dH2, nullptr, H, s));
+    CUDA_TRY(gemm_bf16(gemm, rows, H, O, 0, 1, dYb, O, W3b(), Op, nullptr, 0, dH2, nullptr, H, fault, s));
     CUDA_TRY(launch_relu_mask(rows * H, dH2, H2, dZ2b, s));
-    CUDA_TRY(gemm_bf16(gemm, H, H, rows, 1, 0, H1, H, dZ2b, H, nullptr, 0, G + oW2, nullptr, H, s));
+    CUDA_TRY(gemm_bf16(gemm, H, H, rows, 1, 0, H1, H, dZ2b, H, nullptr, 0, G + oW2, nullptr, H, fault, s));
     CUDA_TRY(launch_colsum(rows, H, dH2, G + ob2, s));
-    CUDA_TRY(gemm_bf16(gemm, rows, H, H, 0, 1, dZ2b, H, W2b(), Hp, nullptr, 0, dH1, nullptr, H, s));
+    CUDA_TRY(gemm_bf16(gemm, rows, H, H, 0, 1, dZ2b, H, W2b(), Hp, nullptr, 0, dH1, nullptr, H, fault, s));
     CUDA_TRY(launch_relu_mask(rows * H, dH1, H1, dZ1b, s));
-    CUDA_TRY(gemm_bf16(gemm, Fpad, H, rows, 1, 0, X, Fpad, dZ1b, H, nullptr, 0, G + oW1, nullptr, H, s));
+    CUDA_TRY(gemm_bf16(gemm, Fpad, H, rows, 1, 0, X, Fpad, dZ1b, H, nullptr, 0, G + oW1, nullptr, H, fault, s));
     CUDA_TRY(launch_colsum(rows, H, dH1, G + ob1, s));
   }
 };
@@ -298,7 +303,7 @@ struct Context {
   double* ydev = nullptr;
   double* bbuf = nullptr;
   double* xbuf = nullptr;
-  double* host_pinned = nullptr;   // 192 doubles: [0,64) scalars and y; [64,128), [128,192) the
+  double* host_pinned = nullptr;   // 192 doubles: [0,63) scalars and y; [63] the network's fault flag; [64,128), [128,192) the
                                    // Hessenberg columns of even and odd Arnoldi steps
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   cudaEvent_t step_done[2] = {};   // end of the last even / odd Arnoldi step launched
@@ -1329,6 +1334,8 @@ int solve_impl(Context& C, const double* b, double* x, double tol, int m, int ma
       loc.restarts += 1;
     }
   }
+  int* mlp_fault = reinterpret_cast<int*>(C.host_pinned + 63);
+  if (C.mlp) CUDA_TRY(cudaMemcpyAsync(mlp_fault, C.mlp->fault, sizeof(int), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaEventRecord(C.ev1, s));
   CUDA_TRY(cudaEventRecord(C.join_out, s));
   CUDA_TRY(cudaStreamWaitEvent(C.stream, C.join_out, 0));
@@ -1341,6 +1348,8 @@ int solve_impl(Context& C, const double* b, double* x, double tol, int m, int ma
     return set_error(SBM_ERR_CUDA, "Gram-Schmidt sweep: staged copies did not complete in bounded time");
   if (tail_fault_take() != 0)
     return set_error(SBM_ERR_CUDA, "V-cycle tail: staging copies did not complete in bounded time");
+  if (C.mlp && *mlp_fault != 0 && tc_fault_take(C.mlp->fault) != 0)
+    return set_error(SBM_ERR_CUDA, "learned correction: a tensor-core wait did not end in bounded time");
   if (status == SBM_ERR_NAN) return set_error(status, "non-finite value in FGMRES");
   if (status == SBM_ERR_NOT_CONVERGED) return set_error(status, "FGMRES did not reach the tolerance");
   return SBM_OK;
@@ -1891,6 +1900,8 @@ int sbm_mlp_create(int dim, int p, int hidden, unsigned long long seed, void* st
     M->Av = M->alloc<float>(M->nparam);
     M->Wb = M->alloc<__nv_bfloat16>(2 * M->weight_elems());
     CUDA_TRY(cudaMemset(M->Wb, 0, 2 * M->weight_elems() * sizeof(__nv_bfloat16)));
+    M->fault = M->alloc<int>(1);
+    CUDA_TRY(cudaMemset(M->fault, 0, sizeof(int)));
     M->loss_part = M->alloc<float>(kLossParts);
     M->loss_tmp = M->alloc<float>(1);
     M->loss_acc = M->alloc<float>(1);
@@ -1947,6 +1958,13 @@ int sbm_mlp_gemm_backend(void* mlp, int backend) {
   return SBM_OK;
 }
 
+int sbm_mlp_wait_limit(void* mlp, int polls) {
+  Mlp* M = mlp_of(mlp);
+  if (!M) return set_error(SBM_ERR_ARG, "null MLP");
+  M->spin = polls < 0 ? kAsyncSpin : std::min((unsigned)polls, kAsyncSpin);
+  return SBM_OK;
+}
+
 int sbm_mlp_forward(void* mlp, const float* X_dev, int rows, float* Y_dev) {
   Mlp* M = mlp_of(mlp);
   if (!M || !X_dev || !Y_dev || rows < 0) return set_error(SBM_ERR_ARG, "bad argument");
@@ -1970,7 +1988,7 @@ int sbm_mlp_gradients(void* mlp, const float* X_dev, const float* T_dev, int row
     M->ensure_batch(rows);
     M->train_pass(X_dev, T_dev, rows);
     const double l = read_loss(*M, rows);
-    if (tc_fault_take() != 0) return set_error(SBM_ERR_CUDA, "a tensor-core GEMM commit did not arrive in time");
+    if (tc_fault_take(M->fault) != 0) return set_error(SBM_ERR_CUDA, "a tensor-core GEMM commit did not arrive in time");
     if (loss) *loss = l;
     if (grad_host) get_packed(*M, M->G, grad_host);
     return SBM_OK;
@@ -2020,7 +2038,7 @@ int sbm_mlp_train(void* mlp, int epochs, int batch, float lr, unsigned long long
       float acc = 0;
       CUDA_TRY(cudaMemcpyAsync(&acc, M->loss_acc, sizeof(float), cudaMemcpyDeviceToHost, M->s));
       CUDA_TRY(cudaStreamSynchronize(M->s));
-      if (tc_fault_take() != 0) return set_error(SBM_ERR_CUDA, "a tensor-core GEMM commit did not arrive in time");
+      if (tc_fault_take(M->fault) != 0) return set_error(SBM_ERR_CUDA, "a tensor-core GEMM commit did not arrive in time");
       last = acc / nbatch;
     }
     if (loss) *loss = last;

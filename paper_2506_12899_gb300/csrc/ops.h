@@ -382,18 +382,20 @@ cudaError_t launch_gemm_bf16(int M, int N, int K, int ta, int tb, const __nv_bfl
                              const __nv_bfloat16* B, int ldb, const float* bias, int relu, float* Cf,
                              __nv_bfloat16* Cb, int ldc, cudaStream_t s);
 // The same GEMM on the tcgen05 tensor cores (tc_gemm.cu): 128 x 128 tiles, FP32 accumulators in
-// tensor memory.  A commit that does not arrive in bounded time sets a flag that tc_fault_take()
-// returns (1) and clears; -1 if it cannot be read.
+// tensor memory.  A commit that does not arrive in bounded time sets *fault (device memory, one flag per
+// network) and leaves zeros; tc_fault_take() returns the flag and clears it, -1 if it cannot be read (call it
+// when the kernels that may set it have completed).
 cudaError_t launch_gemm_tc(int M, int N, int K, int ta, int tb, const __nv_bfloat16* A, int lda,
                            const __nv_bfloat16* B, int ldb, const float* bias, int relu, float* Cf,
-                           __nv_bfloat16* Cb, int ldc, cudaStream_t s);
-int tc_fault_take();
+                           __nv_bfloat16* Cb, int ldc, int* fault, cudaStream_t s);
+int tc_fault_take(int* fault);
 // The whole MLP over one batch of rows in one launch (tc_gemm.cu), for hidden widths that
 // mlp_fused_fits: Y = W3^T relu(W2^T relu(W1^T x + b1) + b2) + b3 for every row x.  Xf: FP32 rows of F
 // features, or (Xf null) Xb: BF16 rows of Fpad.  W1, W2, W3: the core-matrix copies of the weights
 // (MlpWeights); Hp and Op are H and O rounded up to 32.
 // early: the weights were written two or more launches back (they are read before the
-// dependency wait).
+// dependency wait).  spin: polls of a bounded wait; when one runs out *fault is set and the outputs of
+// that CTA's rows are zero (a training pass: undefined).
 struct MlpTile {
   int rows, F, Fpad, H, O, Hp, Op, early;
   bool y_vec;                      // Y is 16-byte aligned
@@ -408,6 +410,8 @@ struct MlpTile {
   float inv_count;
   __nv_bfloat16 *Xs, *H1, *H2, *dY, *dZ2, *dZ1;
   float *bias_part, *loss_part;
+  unsigned spin;
+  int* fault;
 };
 constexpr int kLossParts = 152;    // one per SM
 int mlp_fused_ctas(int rows);
@@ -433,6 +437,7 @@ struct WgradArgs {
   int rows, splits, split_rows;
   size_t part_stride;
   float* part;
+  int* fault;                      // as in MlpTile
 };
 // The products, then G[0, n): the weights' sums over the splits and the biases' over the CTAs of the
 // training pass.

@@ -27,8 +27,6 @@ namespace {
 constexpr int TBM = 128, TBN = 128, TBK = 64;
 constexpr int kTcThreads = 128;
 
-__device__ int g_tc_fault = 0;
-
 // Byte offset of element (row r, k) of a 128 x 64 K-major no-swizzle tile.
 __device__ __forceinline__ uint32_t tile_off(int r, int k) {
   return (uint32_t)(((r >> 3) * 8 + (k >> 3)) * 128 + (r & 7) * 16 + (k & 7) * 2);
@@ -89,7 +87,7 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_tc(int M, int N, int K, con
                                                         int lda, const __nv_bfloat16* __restrict__ B, int ldb,
                                                         const float* __restrict__ bias, int relu,
                                                         float* __restrict__ Cf, __nv_bfloat16* __restrict__ Cb,
-                                                        int ldc) {
+                                                        int ldc, int* fault) {
   // two stages of (A tile, B tile), 32 KB each, in dynamic shared memory (1024-byte aligned)
   extern __shared__ __align__(1024) unsigned char tc_smem[];
   __shared__ __align__(8) unsigned long long bar[2];
@@ -164,7 +162,7 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_tc(int M, int N, int K, con
     failed = !__syncthreads_and(ok);
   }
   if (failed && threadIdx.x == 0) {                  // record it and let the MMAs in flight land
-    atomicExch(&g_tc_fault, 1);
+    atomicExch(fault, 1);
     mbar_wait(&bar[0], phase[0]);
     mbar_wait(&bar[1], phase[1]);
   }
@@ -201,9 +199,9 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_tc(int M, int N, int K, con
         }
       }
     }
-  } else if (K == 0 && m < M) {                      // empty contraction: C = bias (ReLU)
+  } else if (m < M) {                                // empty contraction: C = bias (ReLU); a failed wait: zero
     for (int n = n0; n < n0 + TBN && n < N; ++n) {
-      float v = bias ? bias[n] : 0.f;
+      float v = bias && !failed ? bias[n] : 0.f;
       if (relu) v = fmaxf(v, 0.f);
       if (Cf) Cf[(size_t)m * ldc + n] = v;
       if (Cb) Cb[(size_t)m * ldc + n] = __float2bfloat16_rn(v);
@@ -315,9 +313,12 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_mlp_fused(const __grid_con
   volatile int* stop = &failed;
   // a bounded wait; once one has run out, every role leaves its loop
   auto wait = [&](unsigned long long* bar, unsigned parity) {
-    if (!mbar_wait(bar, parity)) *stop = 1;
+    if (!mbar_wait(bar, parity, P.spin)) *stop = 1;
     return *stop == 0;
   };
+  int issued = 0;                                    // weight chunks copied, or handed to the tensor core, by this thread
+  // (No role starts its bounded polls before the dependency wait: the kernels before this one would count
+  // against the limit.)
 
   if (warp == kFeedWarps) {                          // the weights
     if (lane == 0) {
@@ -326,6 +327,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_mlp_fused(const __grid_con
       bool ok = true;
       for (int tile = blockIdx.x; tile < ntile && ok; tile += gridDim.x)
         for (int i = 0; i < total && ok; ++i, ++g) {
+          if (g == SB && P.early) pdl_wait();        // the ring is full
           if (g >= SB) ok = wait(&empty_b[g % SB], (unsigned)((g / SB - 1) & 1));
           if (!ok) break;
           int at, K, np;
@@ -342,10 +344,12 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_mlp_fused(const __grid_con
             const __nv_bfloat16* W = (layer == 3 ? P.W3 : P.W2) + (size_t)at * kChunkK * 8;
             for (int a = 0; a < Hp / 8; ++a) bulk_load(dst + a * kn * 16, W + (size_t)a * K * 8, (unsigned)kn * 16, bar);
           }
+          issued = g + 1;
         }
     }
   } else if (warp == kFeedWarps + 1) {               // the tensor core
     if (lane == 0) {
+      pdl_wait();
       int ga = 0, gb = 0, layers = 0;                // A and B chunks, layers with an activation tile so far
       bool ok = true;
       for (int tile = blockIdx.x; tile < ntile && ok; tile += gridDim.x)
@@ -369,6 +373,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_mlp_fused(const __grid_con
                      smem_desc(b + ks * 2 * b_lbo, b_lbo, b_sbo), id, at > 0 || ks > 0);
           if (layer == 0) mma_commit(&empty_a[ga++ % SA]);
           mma_commit(&empty_b[gb % SB]);
+          issued = gb + 1;
           if ((at + 1) * kChunkK >= K) mma_commit(&acc_full);
         }
     }
@@ -577,13 +582,18 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_mlp_fused(const __grid_con
         for (int b = gridDim.x; b < kLossParts; ++b) P.loss_part[b] = 0.f;
     }
   }
-  if (failed && threadIdx.x == 0) {                  // record it; copies and MMAs in flight get time to land
-    atomicExch(&g_tc_fault, 1);
-    for (int s = 0; s < SB; ++s)
-      for (unsigned p = 0; p < 2; ++p) mbar_wait(&full_b[s], p, 1u << 16);
-    for (unsigned p = 0; p < 2; ++p) mbar_wait(&acc_full, p, 1u << 16);
+  if (failed) {                                      // record it; copies and MMAs in flight get time to land
+    if (threadIdx.x == 0) atomicExch(P.fault, 1);
+    const bool mma = warp == kFeedWarps + 1;         // (warps 16 and 17 alone have issued any)
+    for (int q = mma ? max(0, issued - 1) : max(0, issued - SB); q < issued; ++q)
+      mbar_wait(mma ? &empty_b[q % SB] : &full_b[q % SB], (unsigned)((q / SB) & 1), 1u << 16);
   }
   __syncthreads();
+  if (!BWD && failed)                                // a defined result: zero outputs for all of this CTA's rows
+    for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+      const size_t beg = (size_t)tile * kTileRows, end = min(beg + kTileRows, (size_t)P.rows);
+      for (size_t q = beg * P.O + threadIdx.x; q < end * P.O; q += kFusedThreads) P.Y[q] = 0.f;
+    }
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
@@ -722,7 +732,7 @@ __global__ void __launch_bounds__(kWgradThreads, 1) k_wgrad(const __grid_constan
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (failed && threadIdx.x == 0) {
-    atomicExch(&g_tc_fault, 1);
+    atomicExch(P.fault, 1);
     for (int s = 0; s < S; ++s)
       for (unsigned p = 0; p < 2; ++p) mbar_wait(&empty[s], p, 1u << 16);
   }
@@ -760,24 +770,25 @@ constexpr size_t kTcSmem = 2 * 2 * (size_t)TBM * TBK * 2;
 
 template <int TA, int TB>
 cudaError_t launch_tc(dim3 grid, int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B,
-                      int ldb, const float* bias, int relu, float* Cf, __nv_bfloat16* Cb, int ldc, cudaStream_t s) {
+                      int ldb, const float* bias, int relu, float* Cf, __nv_bfloat16* Cb, int ldc, int* fault,
+                      cudaStream_t s) {
   const cudaError_t e = cudaFuncSetAttribute(k_gemm_tc<TA, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)kTcSmem);
   if (e != cudaSuccess) return e;
-  k_gemm_tc<TA, TB><<<grid, kTcThreads, kTcSmem, s>>>(M, N, K, A, lda, B, ldb, bias, relu, Cf, Cb, ldc);
+  k_gemm_tc<TA, TB><<<grid, kTcThreads, kTcSmem, s>>>(M, N, K, A, lda, B, ldb, bias, relu, Cf, Cb, ldc, fault);
   return cudaSuccess;
 }
 
 cudaError_t launch_gemm_tc(int M, int N, int K, int ta, int tb, const __nv_bfloat16* A, int lda,
                            const __nv_bfloat16* B, int ldb, const float* bias, int relu, float* Cf,
-                           __nv_bfloat16* Cb, int ldc, cudaStream_t s) {
+                           __nv_bfloat16* Cb, int ldc, int* fault, cudaStream_t s) {
   if (M == 0 || N == 0) return cudaSuccess;
   const dim3 grid((N + TBN - 1) / TBN, (M + TBM - 1) / TBM);
   cudaError_t e;
-  if (!ta && !tb) e = launch_tc<0, 0>(grid, M, N, K, A, lda, B, ldb, bias, relu, Cf, Cb, ldc, s);
-  else if (!ta && tb) e = launch_tc<0, 1>(grid, M, N, K, A, lda, B, ldb, bias, relu, Cf, Cb, ldc, s);
-  else if (ta && !tb) e = launch_tc<1, 0>(grid, M, N, K, A, lda, B, ldb, bias, relu, Cf, Cb, ldc, s);
-  else e = launch_tc<1, 1>(grid, M, N, K, A, lda, B, ldb, bias, relu, Cf, Cb, ldc, s);
+  if (!ta && !tb) e = launch_tc<0, 0>(grid, M, N, K, A, lda, B, ldb, bias, relu, Cf, Cb, ldc, fault, s);
+  else if (!ta && tb) e = launch_tc<0, 1>(grid, M, N, K, A, lda, B, ldb, bias, relu, Cf, Cb, ldc, fault, s);
+  else if (ta && !tb) e = launch_tc<1, 0>(grid, M, N, K, A, lda, B, ldb, bias, relu, Cf, Cb, ldc, fault, s);
+  else e = launch_tc<1, 1>(grid, M, N, K, A, lda, B, ldb, bias, relu, Cf, Cb, ldc, fault, s);
   if (e != cudaSuccess) return e;
   count_launches();
   return cudaGetLastError();
@@ -818,12 +829,12 @@ cudaError_t launch_wgrad(const WgradArgs& P, int n, int ctas, const float* bias_
   return cudaGetLastError();
 }
 
-int tc_fault_take() {
+int tc_fault_take(int* fault) {
   int f = 0;
-  if (cudaMemcpyFromSymbol(&f, g_tc_fault, sizeof(int)) != cudaSuccess) return -1;
+  if (cudaMemcpy(&f, fault, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return -1;
   if (f) {
     const int zero = 0;
-    if (cudaMemcpyToSymbol(g_tc_fault, &zero, sizeof(int)) != cudaSuccess) return -1;
+    if (cudaMemcpy(fault, &zero, sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) return -1;
   }
   return f;
 }
