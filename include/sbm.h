@@ -178,6 +178,11 @@ const char* sbm_last_error(void);
  * contexts; memsets and copies are not counted). */
 long long sbm_kernel_launches(void);
 
+/* 1 if the calling thread's last call with a context or a network launched with programmatic
+ * dependent launch, else 0: a call with a context follows its launch_overlap, a call with a
+ * network alone always overlaps. */
+int sbm_launch_overlap(void);
+
 /* Number of multigrid levels L+1. */
 int sbm_num_levels(const void* ctx, int* out);
 

@@ -26,7 +26,7 @@ ERRORS = {-1: "SBM_ERR_ARG", -2: "SBM_ERR_CUDA", -3: "SBM_ERR_SINGULAR_BLOCK", -
           -5: "SBM_ERR_NAN", -6: "SBM_ERR_GEOMETRY", -7: "SBM_ERR_ALLOC"}
 
 # exported C symbols (checked by the tests against include/sbm.h)
-SYMBOLS = ("sbm_setup", "sbm_setup_host", "sbm_host_apply", "sbm_host_rhs", "sbm_destroy", "sbm_last_error", "sbm_kernel_launches", "sbm_num_levels", "sbm_info", "sbm_layout",
+SYMBOLS = ("sbm_setup", "sbm_setup_host", "sbm_host_apply", "sbm_host_rhs", "sbm_destroy", "sbm_last_error", "sbm_kernel_launches", "sbm_launch_overlap", "sbm_num_levels", "sbm_info", "sbm_layout",
            "sbm_export_geometry", "sbm_rhs", "sbm_apply", "sbm_residual", "sbm_smooth", "sbm_restrict",
            "sbm_prolong_add", "sbm_coarse_solve", "sbm_vcycle", "sbm_dots", "sbm_dots_noalloc", "sbm_gram_schmidt", "sbm_l2_error", "sbm_solve",
            "sbm_solve_host", "sbm_mlp_create", "sbm_mlp_destroy", "sbm_mlp_shape", "sbm_mlp_set_params",
@@ -159,6 +159,11 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
 def kernel_launches() -> int:
     """Kernel launches issued by libsbm since it was loaded."""
     return int(load_library().sbm_kernel_launches())
+
+
+def launch_overlap() -> bool:
+    """Whether the calling thread's last solver or network call launched with overlap (sbm_launch_overlap)."""
+    return bool(load_library().sbm_launch_overlap())
 
 
 def async_wait_selftest(starve: bool, stream=None) -> None:

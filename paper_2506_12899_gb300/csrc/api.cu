@@ -1459,7 +1459,12 @@ Context* ctx_of(void* p) {
   if (C) pdl_enabled() = C->desc.launch_overlap > 0 || (C->desc.launch_overlap == 0 && C->desc.precision == SBM_F32);
   return C;
 }
-Mlp* mlp_of(void* p) { return static_cast<Mlp*>(p); }
+// The network handle of an ABI call of its own: these launches always overlap, whatever context the
+// thread used last (calls that take a context as well follow the context).
+Mlp* mlp_of(void* p) {
+  if (p) pdl_enabled() = true;
+  return static_cast<Mlp*>(p);
+}
 
 int check_level(const Context* C, int& level) {
   if (!C) return set_error(SBM_ERR_ARG, "null context");
@@ -1533,6 +1538,8 @@ void sbm_destroy(void* ctx) { delete ctx_of(ctx); }
 const char* sbm_last_error(void) { return g_last_error.c_str(); }
 
 long long sbm_kernel_launches(void) { return g_kernel_launches.load(); }
+
+int sbm_launch_overlap(void) { return pdl_enabled() ? 1 : 0; }
 
 int sbm_num_levels(const void* ctx, int* out) {
   if (!ctx || !out) return set_error(SBM_ERR_ARG, "null argument");
@@ -2153,7 +2160,7 @@ int sbm_learned_cells(void* ctx, int* n_bnd, int* cells_host) {
 int sbm_collect(void* ctx, void* mlp, int dtype, const void* u0_dev, int n_starts, int n_cycles,
                 long long* n_added) {
   Context* C = ctx_of(ctx);
-  Mlp* M = mlp_of(mlp);
+  Mlp* M = static_cast<Mlp*>(mlp);
   if (C && C->host_only) return set_error(SBM_ERR_ARG, "host-only context");
   if (!C || !M || !u0_dev || n_starts < 0 || n_cycles < 0) return set_error(SBM_ERR_ARG, "bad argument");
   const HostLevel& H = C->lv[C->finest()].H;
@@ -2172,7 +2179,7 @@ int sbm_attach_mlp(void* ctx, void* mlp, float scale, double fallback_rate) {
   Context* C = ctx_of(ctx);
   if (C && C->host_only) return set_error(SBM_ERR_ARG, "host-only context");
   if (!C) return set_error(SBM_ERR_ARG, "null context");
-  Mlp* M = mlp_of(mlp);
+  Mlp* M = static_cast<Mlp*>(mlp);
   if (M) {
     const HostLevel& H = C->lv[C->finest()].H;
     if (M->dim != H.dim || M->p != H.p) return set_error(SBM_ERR_ARG, "MLP shape does not match the finest level");

@@ -275,3 +275,23 @@ def test_training_pass_edges_match_mma_sync(dim, p, hidden, rows):
     ref_loss, ref = gm.gradients(X, T)
     assert abs(loss - ref_loss) <= 2.0 ** -8 * ref_loss
     assert np.linalg.norm(grad - ref) <= 2.0 ** -7 * np.linalg.norm(ref)
+
+
+def test_network_calls_overlap_whatever_solver_was_used_last():
+    """The launch mode of a network's calls is its own: an FP64 solver (no overlap by default) used before
+    on the same thread does not change it, and a call with a solver and a network follows the solver."""
+    import paper_2506_12899_gb300 as S
+    prob = W.disk2d_p1(16, 0)
+    f64, f32 = S.Solver(prob, "f64"), S.Solver(prob, "f32")
+    m = S.Mlp(2, 1, 16)
+    X, T = torch.zeros((3, m.F), device="cuda"), torch.zeros((3, m.O), device="cuda")
+    for solver, mode in ((f64, False), (f32, True)):
+        solver.rhs()
+        assert S.launch_overlap() == mode
+        m.forward(X)
+        assert S.launch_overlap()
+        solver.rhs()
+        m.gradients(X, T)
+        assert S.launch_overlap()
+        solver.attach_mlp(m)
+        assert S.launch_overlap() == mode
