@@ -104,7 +104,10 @@ struct Mlp {
   T* alloc(size_t n) {
     void* q = nullptr;
     cudaError_t e = cudaMalloc(&q, (n ? n : 1) * sizeof(T));
-    if (e != cudaSuccess) throw SetupError{SBM_ERR_ALLOC, std::string("cudaMalloc: ") + cudaGetErrorString(e)};
+    if (e != cudaSuccess) {
+      cudaGetLastError();                            // reported here, not by the next launch
+      throw SetupError{SBM_ERR_ALLOC, std::string("cudaMalloc: ") + cudaGetErrorString(e)};
+    }
     allocs.push_back(q);
     return static_cast<T*>(q);
   }
@@ -170,9 +173,13 @@ struct Mlp {
   }
   void ensure_batch(int B) {
     if (B <= bcap) return;
-    for (void* q : {(void*)Xb, (void*)H1, (void*)H2, (void*)dYb, (void*)dZ2b, (void*)dZ1b, (void*)Tb, (void*)Y,
-                    (void*)dYf, (void*)dH2, (void*)dH1})
+    bcap = 0;                                        // an allocation below may fail: nothing released stays in use
+    auto drop = [this](auto*& q) {
       release(q);
+      q = nullptr;
+    };
+    for (__nv_bfloat16** q : {&Xb, &H1, &H2, &dYb, &dZ2b, &dZ1b}) drop(*q);
+    for (float** q : {&Tb, &Y, &dYf, &dH2, &dH1}) drop(*q);
     Xb = alloc<__nv_bfloat16>((size_t)B * Fpad);     // (rows of the one-launch pass are padded to Hp, Op)
     H1 = alloc<__nv_bfloat16>((size_t)B * Hp);
     H2 = alloc<__nv_bfloat16>((size_t)B * Hp);
@@ -192,6 +199,7 @@ struct Mlp {
     const size_t ncap = std::max(rows, cap * 2);
     __nv_bfloat16* nX = alloc<__nv_bfloat16>(ncap * Fpad);
     float* nT = alloc<float>(ncap * O);
+    int* nidx = alloc<int>(ncap);
     if (count) {
       CUDA_TRY(cudaMemcpyAsync(nX, Xd, count * Fpad * sizeof(__nv_bfloat16), cudaMemcpyDeviceToDevice, s));
       CUDA_TRY(cudaMemcpyAsync(nT, Td, count * O * sizeof(float), cudaMemcpyDeviceToDevice, s));
@@ -202,7 +210,7 @@ struct Mlp {
     release(idx_all);
     Xd = nX;
     Td = nT;
-    idx_all = alloc<int>(ncap);
+    idx_all = nidx;
     cap = ncap;
   }
   // Yout[rows][O] = MLP(X) with the BF16 weights, hidden activations into h1, h2 ([rows][H]).
@@ -374,7 +382,10 @@ struct Context {
     void* p = nullptr;
     if (n == 0) n = 1;
     cudaError_t e = cudaMalloc(&p, n * sizeof(T));
-    if (e != cudaSuccess) throw SetupError{SBM_ERR_ALLOC, std::string("cudaMalloc: ") + cudaGetErrorString(e)};
+    if (e != cudaSuccess) {
+      cudaGetLastError();                            // reported here, not by the next launch
+      throw SetupError{SBM_ERR_ALLOC, std::string("cudaMalloc: ") + cudaGetErrorString(e)};
+    }
     allocs.push_back(p);
     return static_cast<T*>(p);
   }

@@ -295,3 +295,21 @@ def test_network_calls_overlap_whatever_solver_was_used_last():
         assert S.launch_overlap()
         solver.attach_mlp(m)
         assert S.launch_overlap() == mode
+
+
+def test_network_stays_usable_after_a_batch_that_does_not_fit():
+    """A batch whose buffers cannot be allocated (8 TB) is refused with SBM_ERR_ALLOC before any launch; the
+    network then computes smaller batches in buffers of their own, with the same results as before."""
+    import ctypes
+    import paper_2506_12899_gb300 as S
+    m = S.Mlp(3, 3, 264, seed=1)                       # wider than the one-launch kernel: uses the batch buffers
+    g = torch.Generator(device="cuda").manual_seed(0)
+    X = torch.rand((130, m.F), generator=g, device="cuda") - 0.5
+    T = torch.rand((130, m.O), generator=g, device="cuda")
+    y, (loss, grad) = m.forward(X), m.gradients(X, T)
+    code = S.load_library().sbm_mlp_forward(m.h, ctypes.c_void_p(X.data_ptr()), 2_000_000_000,
+                                            ctypes.c_void_p(y.clone().data_ptr()))
+    assert S.ERRORS[code] == "SBM_ERR_ALLOC"
+    assert torch.equal(m.forward(X[:100].contiguous()), y[:100])
+    again = m.gradients(X, T)
+    assert again[0] == loss and np.array_equal(again[1], grad)
