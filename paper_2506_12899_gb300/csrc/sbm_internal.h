@@ -191,7 +191,7 @@ struct TailLevel {
 // so that consecutive cells' words are adjacent (no bank conflicts); cell n_act stays zero and stands
 // for a missing neighbour.  Boundary blocks are padded by 16 bytes for the same reason.
 constexpr int kMaxTailCta = 6;
-constexpr int kTailMats = 136;     // coupling entries (8), interior inverse, interior block
+constexpr int kTailMats = 136;     // coupling entries (8), interior inverse, interior block; the inverse's low part (4: entry i ^ j)
 struct TailLevelDesc {
   int n_act;
   unsigned z, f, binv, aself, mats, rec, ch;   // aself 0: the boundary self blocks stay in global memory (3D: not used)
@@ -204,6 +204,7 @@ struct TailLevelDesc {
 template <typename R>
 struct TailCta {
   int top, pre, post, ssor, n0;    // n0: unknowns of level 0
+  int low;                         // 1: the interior inverses have a low part (2D, finest level p = 1)
   unsigned image_bytes, cinv;      // cinv: the coarse inverse's transpose in the image, 0: not staged
   unsigned vec_bytes;              // the z vectors, from image_bytes on (the f vectors behind them)
   const void* image;
