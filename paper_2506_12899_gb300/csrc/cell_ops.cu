@@ -540,8 +540,9 @@ __device__ int g_tail_fault;
 //     larger than fast diagonalisation had it (disks of 16^2 to 512^2, 25 to 60 of each), with the low part the
 //     error is 3% larger to 6% smaller; a 64^2 V-cycle takes 17.4 instead of 16.2 us.  Below p = 2 and 3 the low
 //     part does not help (error +1 to +3%; -2 to +1% without).
-//   - 3D keeps the operations of the per-level kernels in their order, to the same bits: the long 3D p = 3 solves
-//     (96^3 to 1e-12) end after another number of steps when the rounding of their V-cycle changes;
+//   - 3D keeps the operations of the tail's first form in their order, to the same bits (the tests pin them): the
+//     long 3D p = 3 solves (96^3 to 1e-12) end after another number of steps when the rounding of their V-cycle
+//     changes.  (The per-level kernels round otherwise; they differ in most values by a unit or so.)
 //   - vectors and blocks are laid out free of bank conflicts (TailCta).
 // What is left in 2D is bound by the shared-memory reads of the largest level's phases (the 64^2 level: 850 to
 // 1500 cycles a colour group, 4200 the restriction) and by each thread's chain on the smaller ones (500 to

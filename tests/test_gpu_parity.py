@@ -7,6 +7,8 @@ cell-block inverses (smoother, V-cycle) max(1e-12, n_p eps cond(A_KK)) (see `blo
 1e-10 relative L2 for FGMRES solutions with equal iteration counts.  FP32 tolerances are derived from the
 FP32 unit roundoff (6e-8) times the operation's amplification (stated per test).
 """
+import zlib
+
 import numpy as np
 import pytest
 
@@ -595,3 +597,38 @@ def test_cta_tail_is_as_accurate_as_per_level_launches(n, disks):
             ref = exact.vcycle(r.double())
             err += [((s.vcycle(r).double() - ref).norm() / ref.norm()).item() for s in solvers]
     assert err[0] <= 1.02 * err[1], err / (3 * disks)
+
+
+def _crc(t):
+    return zlib.crc32(t.cpu().numpy().tobytes())
+
+
+def _f32(rng, n):
+    return torch.from_numpy(rng.uniform(-1, 1, n).astype(np.float32)).cuda()
+
+
+@pytest.mark.parametrize("n,p,omega,forward,reverse", [
+    (12, 2, 1.0, 0x4098c97d, 0x9ee396b1), (14, 2, 0.7, 0x272a8730, 0xe95451d6),
+    (10, 3, 0.8, 0xbd815a6d, 0xaa72d618), (12, 3, 1.0, 0xc6263fa2, 0x9ef98190)])
+def test_plane_smoother_keeps_the_bits_of_the_line_form(n, p, omega, forward, reverse):
+    """The 3D p = 2, 3 FP32 sweep adds its terms in the order of the kernel with one lane per x-line that it
+    replaced, to the same bits: CRC-32 of the results, taken with that kernel (commit e2b57b5).  The number of
+    steps of long 3D solves depends on these bits."""
+    import paper_2506_12899_gb300 as S
+    a = S.Solver(W.sphere3d(n, 2, 1).replace(p=p, coarsest_n=4, omega=omega, omega_p3=omega), "f32")
+    rng = np.random.default_rng(n)
+    f, u = _f32(rng, a.n_dof()), _f32(rng, a.n_dof())
+    assert _crc(a.smooth(f, u.clone())) == forward
+    assert _crc(a.smooth(f, u.clone(), reverse=True)) == reverse
+
+
+@pytest.mark.parametrize("n,geometry,kw,crc", [
+    (8, 1, dict(), 0x24558b36), (16, 2, dict(), 0xc9b6694c), (16, 0, dict(omega=0.9, post_smooth=2), 0x596c327b),
+    (16, 3, dict(ssor_each=1), 0xd8f94f8d), (32, 1, dict(pre_smooth=0, post_smooth=2), 0x475e82af),
+    (32, 0, dict(), 0xed805dea)])
+def test_3d_tail_keeps_its_bits(n, geometry, kw, crc):
+    """V-cycles of 3D p = 1 spheres, inside the one-CTA tail (8^3, 16^3) and above it, to the bits of the tail's
+    first form (CRC-32 of the results, commit e2b57b5), for the same reason."""
+    import paper_2506_12899_gb300 as S
+    a = S.Solver(W.sphere3d(n, 1, geometry).replace(**kw), "f32")
+    assert _crc(a.vcycle(_f32(np.random.default_rng(n), a.n_dof()))) == crc
