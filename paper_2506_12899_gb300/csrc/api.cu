@@ -43,6 +43,7 @@ struct DevLevel {
   int* children = nullptr;
   double* coarse_inv = nullptr;
   LevelParams<double> P64{};
+  LevelParams<double> V64{};         // P64 as the FP64 V-cycle uses it (with the self blocks on every level)
   LevelParams<float> P32{};
   LevelParams<dfl> Pdf{};         // double-float operator constants (finest level, thread-per-cell shapes)
   dfl* dhat_df = nullptr;
@@ -401,7 +402,7 @@ struct Context {
 template <typename R>
 const LevelParams<R>& params(const DevLevel& L);
 template <>
-const LevelParams<double>& params<double>(const DevLevel& L) { return L.P64; }
+const LevelParams<double>& params<double>(const DevLevel& L) { return L.V64; }
 template <>
 const LevelParams<float>& params<float>(const DevLevel& L) { return L.P32; }
 template <typename R>
@@ -568,6 +569,35 @@ void estimate_lambda_max(Context& C) {
   }
 }
 
+constexpr int kSelfNp = 27;           // largest cell whose FP64 self block is stored (3D p = 2: 5.8 KB)
+
+// The boundary blocks of a level by entry for the thread-per-cell kernels (LevelParams::binvS, aselfS), once.
+template <typename R>
+void upload_by_entry(Context& C, DevLevel& L, LevelParams<R>& P) {
+  const HostLevel& H = L.H;
+  const int min_cells = C.desc.cell_kernel_min_cells;
+  if (!cell_smoother(H.dim, H.p) || H.n_bnd == 0 || P.binvS || min_cells < 0 || (sizeof(R) == 8 && min_cells == 0)) return;
+  const size_t ld = ((size_t)H.n_bnd + 31) / 32 * 32, nq = (size_t)H.np * H.np;
+  auto by_entry = [&](const std::vector<double>& blocks) {
+    std::vector<R> s(nq * ld, R(0));
+    for (int b = 0; b < H.n_bnd; ++b)
+      for (size_t q = 0; q < nq; ++q) s[q * ld + b] = (R)blocks[b * nq + q];
+    return s;
+  };
+  if (sizeof(R) == 4 && H.p == 1 && H.dim == 2) P.aselfS = C.upload(by_entry(H.aselfT));
+  P.bnd_ld = (int)ld;
+  P.binvS = C.upload(by_entry(H.binvT));
+}
+
+// What the V-cycle of one precision needs beyond the level's parameters: at set-up for the context's own
+// precision, with the first V-cycle for the other.  (Uploaded for both, the blocks took 5.8 KB per boundary cell
+// of a 3D p = 2 level and a few per cent of the set-up time in contexts that never read them.)
+void ensure_blocks(Context& C, DevLevel& L, float) { upload_by_entry<float>(C, L, L.P32); }
+void ensure_blocks(Context& C, DevLevel& L, double) {
+  upload_by_entry<double>(C, L, L.V64);
+  if (!L.V64.aselfT && L.H.n_bnd > 0 && L.H.np <= kSelfNp) L.V64.aselfT = C.upload(self_blocks(L.H));
+}
+
 Context* build_context(const sbm_setup_desc& d, bool device) {
   validate(d);
   auto C = std::make_unique<Context>();
@@ -584,7 +614,11 @@ Context* build_context(const sbm_setup_desc& d, bool device) {
     DevLevel L;
     if (np.first != counts_n) counts.clear();
     counts_n = np.first;
-    L.H = build_level(d, np.first, np.second, device, &counts);
+    // self blocks: kept where they go to the device at set-up (FP64 contexts: every level; others: the finest, for
+    // the true residual) and on 2D p = 1 levels (the FP32 V-cycle); self_blocks() computes them elsewhere
+    const int n1 = np.second + 1, ndof = d.dim == 2 ? n1 * n1 : n1 * n1 * n1;
+    const bool stored = ndof <= kSelfNp && (d.precision == SBM_F64 || np == seq.back());
+    L.H = build_level(d, np.first, np.second, device, &counts, device && (stored || (d.dim == 2 && np.second == 1)));
     if (L.H.n_act == 0) {
       C->lv.clear();                       // an empty level: everything coarser is dropped
       continue;
@@ -610,21 +644,10 @@ Context* build_context(const sbm_setup_desc& d, bool device) {
     L.P64 = make_params<double>(L, L.dhat64, L.binv64);
     L.P32 = make_params<float>(L, L.dhat32, L.binv32);
     L.P64.ordering = L.P32.ordering = d.ordering;
-    if (!L.H.aselfT.empty()) L.P64.aselfT = C->upload(L.H.aselfT);
-    if (cell_smoother(L.H.dim, L.H.p) && L.H.n_bnd > 0) {   // the blocks by entry (thread-per-cell kernels)
-      const size_t ld = ((size_t)L.H.n_bnd + 31) / 32 * 32, nq = (size_t)L.H.np * L.H.np;
-      auto by_entry = [&](const std::vector<double>& blocks) {
-        std::vector<double> s(nq * ld, 0.0);
-        for (int b = 0; b < L.H.n_bnd; ++b)
-          for (size_t q = 0; q < nq; ++q) s[q * ld + b] = blocks[b * nq + q];
-        return s;
-      };
-      const std::vector<double> bs = by_entry(L.H.binvT);
-      L.P64.bnd_ld = L.P32.bnd_ld = (int)ld;
-      if (d.cell_kernel_min_cells >= 0) L.P32.binvS = C->upload(to_f32(bs));
-      if (d.cell_kernel_min_cells > 0) L.P64.binvS = C->upload(bs);
-      if (d.cell_kernel_min_cells >= 0 && L.H.p == 1 && L.H.dim == 2) L.P32.aselfS = C->upload(to_f32(by_entry(L.H.aselfT)));
-    }
+    if (!L.H.aselfT.empty() && (d.precision == SBM_F64 || &L == &C->lv.back())) L.P64.aselfT = C->upload(L.H.aselfT);
+    if (L.H.dim == 3 || L.H.p > 1) std::vector<double>().swap(L.H.aselfT);
+    if (d.precision == SBM_F64) upload_by_entry<double>(*C, L, L.P64);
+    else upload_by_entry<float>(*C, L, L.P32);
     if (&L == &C->lv.back()) {                     // Arnoldi operator in double-float
       std::vector<dfl> dh(L.H.dhat.size());
       for (size_t i = 0; i < dh.size(); ++i) dh[i] = dfl(L.H.dhat[i]);
@@ -667,6 +690,7 @@ Context* build_context(const sbm_setup_desc& d, bool device) {
     L.Pdf.cell_min = L.P32.cell_min;               // the double-float operator follows the FP32 choice
     // staged thread-per-cell kernels (FP32): launches over at least staged_min cells
     L.P32.staged_min = d.staged_min_cells == 0 ? 0 : (d.staged_min_cells < 0 ? 0 : d.staged_min_cells);
+    L.V64 = L.P64;
   }
   for (size_t l = 1; l < C->lv.size(); ++l) {
     C->lv[l].T64 = make_transfer<double>(C->lv[l - 1], C->lv[l]);
@@ -839,6 +863,7 @@ template <typename R>
 void ensure_work(Context& C) {
   const int pi = prec_index<R>();
   if (C.work_ready[pi]) return;
+  for (auto& L : C.lv) ensure_blocks(C, L, R(0));
   // one allocation for every level's vectors, each on a 256-byte boundary
   const int nvec = C.desc.smoother == 0 ? 3 : (C.desc.smoother == 2 ? 5 : 4);
   auto padded = [](const DevLevel& L) { return ((size_t)L.H.n_dof() + 63) / 64 * 64; };

@@ -42,7 +42,7 @@ struct HostLevel {
   int colour_start[9] = {}, colour_nbnd[8] = {}, bstart[8] = {};
   std::vector<double> dhat;         // [n_bnd][nslot][dim][nq]  d / h (zero on non-surrogate slots)
   std::vector<double> binvT;        // [n_bnd][np][np]  (A_KK^{-1})^T: element (j, i) at j*np + i
-  std::vector<double> aselfT;       // [n_bnd][np][np] (A_KK)^T in the same form (levels with np <= 27)
+  std::vector<double> aselfT;       // [n_bnd][np][np] (A_KK)^T in the same form (where build_level was asked to keep it)
   std::vector<int> parent_code;     // [n_act] (parent compact index << 3) | child bits, or -1
   std::vector<int> children;        // [2^dim][n_act] compact index of child in the next finer level
   std::vector<int> sf_cell, sf_slot;
@@ -76,7 +76,8 @@ struct SetupError {
 // counts_cache: the sub-cell sample counts of the volume fractions on an n-cell mesh, shared by the
 // levels of one mesh size (the p-levels): used when it holds n^dim entries, else filled.
 HostLevel build_level(const sbm_setup_desc& d, int n, int p, bool device = false,
-                      std::vector<int>* counts_cache = nullptr);
+                      std::vector<int>* counts_cache = nullptr, bool keep_self = false);
+std::vector<double> self_blocks(const HostLevel& L);
 // Device set-up kernels (geometry_ops.cu); throw SetupError on CUDA failures.
 void device_volume_counts(const sbm_setup_desc& d, int n, double h, int s, std::vector<int>& counts);
 void device_closest_points(const sbm_setup_desc& d, const std::vector<double>& samples, const std::vector<double>& X,
@@ -132,8 +133,9 @@ struct LevelParams {
   // (FP32 p = 1 levels: k_resid_restrict_h_cell; null elsewhere)
   const R* aselfS;
   int bnd_ld;
-  // h^(d-2) A_KK of the boundary cells, transposed, block b at b * np * np (FP64 levels with np <= 27; null elsewhere:
-  // the thread-per-DoF kernels then evaluate the surrogate-face terms)
+  // h^(d-2) A_KK of the boundary cells, transposed, block b at b * np * np (FP64, np <= 27: the levels of an FP64
+  // V-cycle and every finest level; null elsewhere: the thread-per-DoF kernels then evaluate the surrogate-face
+  // terms)
   const R* aselfT;
   // dense self blocks h^(d-2) A_KK of the boundary cells (Eqs. 10, 7), column j at bself_ld * b + np * j
   // (double-float operator of a 3D p = 1 finest level only; null elsewhere)

@@ -415,7 +415,8 @@ void cell_self_apply(const HostLevel& L, int a, int bidx, const double* u, doubl
 }
 
 // ------------------------------------------------------------------------------ level set-up
-HostLevel build_level(const sbm_setup_desc& d, int n, int p, bool device, std::vector<int>* counts_cache) {
+HostLevel build_level(const sbm_setup_desc& d, int n, int p, bool device, std::vector<int>* counts_cache,
+                      bool keep_self) {
   HostLevel L;
   L.dim = d.dim;
   L.n = n;
@@ -695,7 +696,6 @@ HostLevel build_level(const sbm_setup_desc& d, int n, int p, bool device, std::v
 
   // dense blocks A_KK of boundary cells (Eq. 14) and their inverses, stored transposed
   L.binvT.assign((size_t)L.n_bnd * np * np, 0.0);
-  const bool keep_self = np <= 27;
   if (keep_self) L.aselfT.assign((size_t)L.n_bnd * np * np, 0.0);
   std::vector<double> ratio(L.n_bnd, 1.0);
   parallel_for(L.n_bnd, [&](int b0, int b1) {
@@ -745,6 +745,25 @@ void host_apply_level(const HostLevel& L, const double* x, double* y) {
       }
     }
   });
+}
+
+// (A_KK)^T of the boundary cells of a built level, as build_level keeps them.
+std::vector<double> self_blocks(const HostLevel& L) {
+  const int np = L.np;
+  std::vector<double> out((size_t)L.n_bnd * np * np, 0.0);
+  std::vector<int> cell(L.n_bnd);
+  for (int c = 0; c < L.ncol; ++c)
+    for (int off = 0; off < L.colour_nbnd[c]; ++off) cell[L.bstart[c] + off] = L.colour_start[c] + off;
+  parallel_for(L.n_bnd, [&](int b0, int b1) {
+    std::vector<double> e(np);
+    for (int b = b0; b < b1; ++b)
+      for (int j = 0; j < np; ++j) {
+        std::fill(e.begin(), e.end(), 0.0);
+        e[j] = 1.0;
+        cell_self_apply(L, cell[b], b, e.data(), &out[((size_t)b * np + j) * np]);
+      }
+  });
+  return out;
 }
 
 void link_levels(HostLevel& C, HostLevel& F) {

@@ -632,3 +632,31 @@ def test_3d_tail_keeps_its_bits(n, geometry, kw, crc):
     import paper_2506_12899_gb300 as S
     a = S.Solver(W.sphere3d(n, 1, geometry).replace(**kw), "f32")
     assert _crc(a.vcycle(_f32(np.random.default_rng(n), a.n_dof()))) == crc
+
+
+@pytest.mark.parametrize("name", ["sphere3d_p3", "star2d_p2", "sphere3d_p1"])
+def test_vcycle_blocks_are_held_for_the_precisions_used(name):
+    """FP64 self blocks of the levels below the finest belong to the FP64 V-cycle: an FP32 solver holds them only
+    from its first FP64 V-cycle on.  Either solver runs V-cycles of either precision to the same bits."""
+    import paper_2506_12899_gb300 as S
+    prob = {"sphere3d_p3": W.sphere3d(40, 2, 0).replace(p=3, coarsest_n=4), "star2d_p2": W.star2d_p2(64, 0),
+            "sphere3d_p1": W.sphere3d(16, 1, 0)}[name]
+
+    def held(precision):                               # bytes of device memory a set-up takes
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        s = S.Solver(prob, precision)
+        return s, free - torch.cuda.mem_get_info()[0]
+
+    for precision in ("f32", "f64"):                   # code is loaded
+        held(precision)[0].close()
+    a, small = held("f32")
+    b, large = held("f64")
+    blocks = 0
+    for l in range(a.num_levels - 1):
+        info = a.info(l)
+        blocks += info["n_boundary"] * (info["n_dof"] // info["n_active"]) ** 2 * 8
+    assert small <= large - blocks + (4 << 20), (small, large, blocks)   # allocations come in 2 MB pieces
+    r = _f32(np.random.default_rng(1), a.n_dof())
+    for x in (r, r.double()):
+        assert torch.equal(a.vcycle(x), b.vcycle(x))
