@@ -313,3 +313,51 @@ def test_network_stays_usable_after_a_batch_that_does_not_fit():
     assert torch.equal(m.forward(X[:100].contiguous()), y[:100])
     again = m.gradients(X, T)
     assert again[0] == loss and np.array_equal(again[1], grad)
+
+
+_ROWS_CASES = [("star", 64, False), ("star", 200, False), ("star", 256, False), ("sphere", 32, True), ("sphere", 200, True)]
+
+
+def _rows_problem(name):
+    return W.random_star2d_p3(64, 1002) if name == "star" else W.sphere3d(128, 1, 0)
+
+
+@pytest.mark.parametrize("name,hidden,two_tiles", _ROWS_CASES)
+def test_attached_correction_matches_mma_sync(name, hidden, two_tiles):
+    """The one-launch pass over BF16 feature rows, as an attached V-cycle runs it, against the mma.sync layers:
+    widths below and above 128, and more rows than one 128-row tile per SM.  Same BF16 products, FP32 sums in
+    another order, so one BF16 unit (2^-8) of one hidden value."""
+    import paper_2506_12899_gb300 as S
+    a = S.Solver(_rows_problem(name), "f32")
+    assert (len(a.learned_cells()) > 152 * 128) == two_tiles
+    r = torch.rand(a.n_dof(), generator=torch.Generator(device="cuda").manual_seed(hidden), device="cuda") - 0.5
+    plain = a.vcycle(r)
+    m = S.Mlp(a.prob.dim, a.prob.p, hidden, seed=7)
+    a.attach_mlp(m, scale=1.0)
+    z = a.vcycle(r) - plain
+    m.gemm_backend(1)
+    ref = a.vcycle(r) - plain
+    assert ref.norm() > 0 and (z - ref).norm() <= 2.0 ** -8 * ref.norm()
+
+
+@pytest.mark.parametrize("name,hidden,two_tiles", _ROWS_CASES)
+def test_training_on_stored_rows_matches_mma_sync(name, hidden, two_tiles):
+    """One training step over the whole stored set (BF16 rows) against the mma.sync layers.  The loss of the
+    step differs by BF16 rounding (2^-8).  Adam's first step is lr times the gradient's sign: an entry whose
+    gradient is below its rounding error (2^-7 of the gradients' size, as in the pass with FP32 rows) may
+    change sign; at most 5% of them are that small, so the steps' cosine is at least 0.9."""
+    import paper_2506_12899_gb300 as S
+    a = S.Solver(_rows_problem(name), "f32")
+    u0 = torch.rand((1, a.n_dof()), generator=torch.Generator(device="cuda").manual_seed(hidden), device="cuda") - 0.5
+    step, loss = [], []
+    for backend in (0, 1):
+        m = S.Mlp(a.prob.dim, a.prob.p, hidden, seed=7)
+        rows = a.collect(m, u0, 1)
+        assert (rows > 152 * 128) == two_tiles
+        m.gemm_backend(backend)
+        before = m.get_params()
+        loss.append(m.train(epochs=1, batch=rows, lr=1e-3, seed=0))
+        step.append((m.get_params() - before).astype(np.float64))
+    assert abs(loss[0] - loss[1]) <= 2.0 ** -8 * loss[1]
+    cosine = step[0] @ step[1] / (np.linalg.norm(step[0]) * np.linalg.norm(step[1]))
+    assert cosine >= 0.9, cosine
