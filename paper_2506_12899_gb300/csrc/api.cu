@@ -752,7 +752,7 @@ size_t build_tail_cta(Context& C, int top, TailCta<R>& T) {
       for (; k < 3; ++k) end[k] = n;
       D[l].grp[g] = {end[0], end[1], end[2], first[0], first[1], first[2]};
     }
-    D[l].mats = take(kTailMats * sizeof(R));
+    D[l].mats = take(tail_mats(dim) * sizeof(R));
     D[l].binv = take(H.n_bnd * blk);
     D[l].rec = take((size_t)H.n_act * 16);
     if (l >= 1) D[l].ch = take((size_t)ncol * C.lv[l - 1].H.n_act * 2);
@@ -785,15 +785,15 @@ size_t build_tail_cta(Context& C, int top, TailCta<R>& T) {
   std::memcpy(image.data(), D.data(), D.size() * sizeof(TailLevelDesc));
   for (int l = 0; l <= top; ++l) {
     const HostLevel& H = C.lv[l].H;
-    // couplings h^(d-2) w B (p = 1: every face point has the weight w), the transposed inverse (by fast
-    // diagonalisation) and self block of an interior cell: FP64, then rounded
+    // couplings h^(d-2) w B (p = 1: every face point has the weight w); 2D: the transposed inverse (by fast
+    // diagonalisation) and self block of an interior cell.  FP64, then rounded
     R* M = reinterpret_cast<R*>(&image[D[l].mats]);
     const double hs = std::pow(H.h, dim - 2), wt = dim == 2 ? H.B.w[0] : H.B.w[0] * H.B.w[0];
     for (int q = 0; q < 4; ++q) {
       M[q] = dim == 2 ? (R)(hs * wt * H.Bpm[q]) : (R)H.Bpm[q];   // 3D: weighted in the kernel
       M[4 + q] = dim == 2 ? (R)(hs * wt * H.Bmp[q]) : (R)H.Bmp[q];
     }
-    for (int i = 0; i < np; ++i)
+    for (int i = 0; i < np && dim == 2; ++i)
       for (int j = 0; j < np; ++j) {
         double inv = 0, self = 0;
         for (int m = 0; m < np; ++m) {

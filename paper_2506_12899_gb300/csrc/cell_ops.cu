@@ -114,7 +114,7 @@ __device__ __forceinline__ void dense_apply(const R (&B)[NN], const R (&t)[NP], 
 // cells: the neighbours, then the dense inverse.  PRE: the inverse (set-up data) is read into registers
 // before the dependency wait.  It is read by entry (binvS), 128 contiguous bytes per warp and entry; from
 // the cells' own blocks every one of the (p+1)^(2d) loads touched 32 lines.  V-cycle of the 512^2 p = 2 star
-// 107 -> 96 us, of the 64^3 p = 1 sphere 108 -> 79 us.  PRE is for launches of up to 32 warps per SM (32-thread
+// 107 -> 96 us, of the 64^3 p = 1 sphere 29 us less (89 now).  PRE is for launches of up to 32 warps per SM (32-thread
 // blocks) and (p+1)^d <= 9 FP32 values; larger launches hide the reads behind other warps.
 template <int D, int N1, typename R, bool PRE>
 __global__ void __launch_bounds__(PRE ? 32 : kCellThreads) k_smooth_cell(const __grid_constant__ LevelParams<R> P,
@@ -229,8 +229,9 @@ __device__ __forceinline__ R h_weight(const TransferParams<R>& T, int o, int i, 
 //
 // PRE (as in k_smooth_cell): with SM0 the coarse cells' inverses, and in 2D the children's self blocks instead
 // of their surrogate-face terms, are read before the dependency wait: V-cycle of the 512^2 p = 2 star 95.7 ->
-// 94.1 us.  (3D keeps the order of its operations, see k_vcycle_tail_cta.  Not at 2D p = 2, k_resid_restrict_p_cell: 81 registers of block made that V-cycle 1.8 us longer; nor after the
-// wait in the operator: 44 -> 46 us at 2048^2 p = 2.)
+// 94.1 us.  (3D keeps the order of its operations, see k_vcycle_tail_cta.  Not at 2D p = 2,
+// k_resid_restrict_p_cell: 81 registers of block made that V-cycle 1.8 us longer; nor after the wait in the
+// operator: 44 -> 46 us at 2048^2 p = 2.)
 template <int D, typename R, bool SM0, bool PRE>
 __global__ void __launch_bounds__(PRE ? 32 : kCellThreads) k_resid_restrict_h_cell(const __grid_constant__ LevelParams<R> P,
                                                                         const __grid_constant__ TransferParams<R> T,
@@ -864,20 +865,20 @@ __global__ void __launch_bounds__(kTailCtaThreads, 1) k_vcycle_tail_cta(const __
 #pragma unroll
             for (int j = 0; j < NP; ++j) r[j] = out[j];
           } else {
-          if (aself) block(b == 0xffffu ? M + 8 + NP * NP : reinterpret_cast<const R*>(tcta_smem + aself + b * BLK), u, R(-1), r);
-          else block(b == 0xffffu ? M + 8 + NP * NP : TP.aselfT[l] + b * (NP * NP), u, R(-1), r);
-          couple(q, z, n, bc, r);
+            if (aself) block(b == 0xffffu ? M + 8 + NP * NP : reinterpret_cast<const R*>(tcta_smem + aself + b * BLK), u, R(-1), r);
+            else block(b == 0xffffu ? M + 8 + NP * NP : TP.aselfT[l] + b * (NP * NP), u, R(-1), r);
+            couple(q, z, n, bc, r);
 #pragma unroll
-          for (int dir = 0; dir < D; ++dir) {
-            const bool hi = (o >> dir) & 1;
+            for (int dir = 0; dir < D; ++dir) {
+              const bool hi = (o >> dir) & 1;
 #pragma unroll
-            for (int tl = 0; tl < NP / 2; ++tl) {
-              const int i0 = dof<D, 2>(dir, 0, tl), i1 = dof<D, 2>(dir, 1, tl);
-              const R e0 = r[i0], e1 = r[i1];
-              r[i0] = (hi ? P1[0] : P0[0]) * e0 + (hi ? P1[2] : P0[2]) * e1;
-              r[i1] = (hi ? P1[1] : P0[1]) * e0 + (hi ? P1[3] : P0[3]) * e1;
+              for (int tl = 0; tl < NP / 2; ++tl) {
+                const int i0 = dof<D, 2>(dir, 0, tl), i1 = dof<D, 2>(dir, 1, tl);
+                const R e0 = r[i0], e1 = r[i1];
+                r[i0] = (hi ? P1[0] : P0[0]) * e0 + (hi ? P1[2] : P0[2]) * e1;
+                r[i1] = (hi ? P1[1] : P0[1]) * e0 + (hi ? P1[3] : P0[3]) * e1;
+              }
             }
-          }
           }
         }
         // the sum over the children: at each exchange a lane keeps half of the values
@@ -1021,12 +1022,12 @@ cudaError_t launch_resid_restrict_h_cell(int dim, const LevelParams<R>& P, const
   const bool sm0 = Pc != nullptr && zc != nullptr;
   const LevelParams<R>& Q = sm0 ? *Pc : P;
   constexpr bool kPre = sizeof(R) == 4;
-  const bool pre = kPre && bs == 32 && (dim == 3 || P.aselfS) && (!sm0 || Q.binvS);
+  const bool pre = kPre && bs == 32 && (dim == 3 ? sm0 : P.aselfS != nullptr) && (!sm0 || Q.binvS);
 #define SBM_RRHC(D)                                                                                               \
   {                                                                                                               \
     if (sm0 && pre) SBM_PDL((k_resid_restrict_h_cell<D, R, true, kPre>), g, bs, 0, s, P, T, u, f, rc, early, Q, zc); \
     else if (sm0) SBM_PDL((k_resid_restrict_h_cell<D, R, true, false>), g, bs, 0, s, P, T, u, f, rc, early, Q, zc);  \
-    else if (pre) SBM_PDL((k_resid_restrict_h_cell<D, R, false, kPre>), g, bs, 0, s, P, T, u, f, rc, early, Q, zc);  \
+    else if (pre) SBM_PDL((k_resid_restrict_h_cell<D, R, false, kPre && D == 2>), g, bs, 0, s, P, T, u, f, rc, early, Q, zc); \
     else SBM_PDL((k_resid_restrict_h_cell<D, R, false, false>), g, bs, 0, s, P, T, u, f, rc, early, Q, zc);          \
   }
   if (dim == 2) SBM_RRHC(2)

@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(256) k_restrict(const __grid_constant__ Transf
   rc[(size_t)cc * NPC + j] = sum;
 }
 
-// Prolongation uf += P ec (Eq. 17) per fine dof; fine cells without an active parent get 0.
+// The h-prolongation uf += P ec (Eq. 17) per fine dof; fine cells without an active parent get 0.
 template <int D, int NF, int NC, typename R>
 __global__ void __launch_bounds__(256) k_prolong(const __grid_constant__ TransferParams<R> T,
                                                  const R* __restrict__ ec, R* __restrict__ uf, int early) {
@@ -555,25 +555,18 @@ __global__ void __launch_bounds__(256) k_prolong(const __grid_constant__ Transfe
   constexpr int NPC = D == 2 ? NC * NC : NC * NC * NC;
   const size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int a = (int)(gid / NPF), i = (int)(gid % NPF);
-  const int code = T.hmode && a < T.n_act_f ? T.parent_code[a] : 0;   // set-up data: before the wait
+  const int code = a < T.n_act_f ? T.parent_code[a] : 0;   // set-up data: before the wait
   R uv = 0;
   if (early && a < T.n_act_f && code >= 0) uv = __ldcg(uf + (size_t)a * NPF + i);   // uf two launches back (L2)
   pdl_wait();
   pdl_trigger();
   if (a >= T.n_act_f) return;
   if (!early && code >= 0) uv = uf[(size_t)a * NPF + i];
-  int par;
-  const R *P0, *P1, *P2;
-  if (T.hmode) {
-    if (code < 0) return;
-    par = code >> 3;
-    P0 = T.Ph[code & 1];
-    P1 = T.Ph[(code >> 1) & 1];
-    P2 = T.Ph[(code >> 2) & 1];
-  } else {
-    par = a;
-    P0 = P1 = P2 = T.Pp;
-  }
+  if (code < 0) return;
+  const int par = code >> 3;
+  const R* P0 = T.Ph[code & 1];
+  const R* P1 = T.Ph[(code >> 1) & 1];
+  const R* P2 = T.Ph[(code >> 2) & 1];
   const int i0 = i % NF, i1 = (i / NF) % NF, i2 = D == 3 ? i / (NF * NF) : 0;
   const R* e = ec + (size_t)par * NPC;
   R s2 = 0;

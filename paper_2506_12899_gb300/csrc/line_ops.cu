@@ -15,9 +15,10 @@
 // the 1D matrices come from the kernel's parameter block.  Surrogate faces (Eq. 7) follow in three
 // barrier-separated phases per face slot: the cell's lanes take the N1^2 points of the face (trace
 // and normal derivative, then the extended value), then every lane adds the face terms at its own
-// values.  The smoother's fast diagonalisation contracts x on the thread's line and y, z after
-// exchanges through shared memory; a cell's lanes lie in one warp, so those exchanges need only
-// warp barriers.
+// values.  A cell's lanes lie in one warp, so exchanges between them need only warp barriers.
+//
+// The smoother takes this form on boundary cells alone, for the couplings; its interior cells have one
+// lane per x-y plane (smooth_planes).
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -437,9 +438,9 @@ __device__ __forceinline__ void plane_apply(const float* M, int dir, float (&v)[
 // cell and of every neighbour into registers, contracts x and y there and exchanges z contributions with the
 // cell's other lanes.  With one lane per line and everything in shared memory, the shared-memory reads
 // bound the launch (32 16-byte reads per lane and 3 cells per warp at p = 2); here it is 108 exchanges for
-// 10 cells.  The terms are added in the same order as there, to the same bits.  (Exchanging products instead
-// of planes takes half the exchanges, 52 instead of 55 us for a 112^3 p = 2 sweep, but rounds otherwise, and
-// the long 96^3 p = 3 solve to 1e-12 then ends after another number of steps.)
+// 10 cells.  The terms are added in the same order as there, to the same bits (the tests pin them).
+// (Exchanging products instead of planes takes half the exchanges, 52 instead of 55 us for a 112^3 p = 2
+// sweep, but rounds otherwise, and the long 96^3 p = 3 solve to 1e-12 then ends after another number of steps.)
 // 128 threads; blk: the block's number in its segment.  112^3 p = 2 sweep 97.6 -> 55.2 us,
 // 96^3 p = 3 solve 83.1 -> 73.4 ms.
 template <int N1>

@@ -193,10 +193,12 @@ struct TailLevel {
 // so that consecutive cells' words are adjacent (no bank conflicts); cell n_act stays zero and stands
 // for a missing neighbour.  Boundary blocks are padded by 16 bytes for the same reason.
 constexpr int kMaxTailCta = 6;
-constexpr int kTailMats = 136;     // coupling entries (8), interior inverse, interior block; the inverse's low part (4: entry i ^ j)
+// entries of a level's matrices: the couplings (8); in 2D also the interior inverse, the interior block and the
+// inverse's low part (4: entry i ^ j)
+constexpr int tail_mats(int dim) { return dim == 2 ? 8 + 2 * 16 + 4 : 8; }
 struct TailLevelDesc {
   int n_act;
-  unsigned z, f, binv, aself, mats, rec, ch;   // aself 0: the boundary self blocks stay in global memory (3D: not used)
+  unsigned z, f, binv, aself, mats, rec, ch;   // aself 0: the boundary self blocks stay in global memory (3D: none)
   // cell idx (0 <= idx < end2) of a colour group: idx + first0 below end0, + first1 below end1, + first2
   // below end2 (a group has up to three colours, each a range of cells)
   struct Group {

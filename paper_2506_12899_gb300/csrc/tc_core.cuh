@@ -1,4 +1,4 @@
-// Device helpers shared by the tcgen05 kernels (tc_gemm.cu, mlp_fused.cu): shared-memory operand
+// Device helpers shared by the tcgen05 kernels (tc_gemm.cu): shared-memory operand
 // tiles without swizzle, their asynchronous staging, instruction descriptors and accumulator loads.
 // Included inside namespace sbm { namespace { ... } }.
 //
