@@ -349,8 +349,10 @@ int sbm_mlp_get_params(const void* mlp, float* params_host);
  * accumulators in tensor memory), 1 the warp-level mma.sync kernel.  Both compute the same
  * BF16 x BF16 -> FP32 products (summation order differs).  Every wait of the tcgen05 kernels is
  * bounded.  One that runs out sets a flag of this network: its outputs are zero (a correction of zero
- * inside sbm_vcycle), and the next call that synchronises and uses the network (sbm_mlp_gradients,
- * sbm_mlp_train, sbm_solve with the network attached) returns SBM_ERR_CUDA and clears the flag. */
+ * inside sbm_vcycle; hidden widths above 256 run layer by layer, and then the layer where it happened
+ * is zero), and the next call that synchronises and uses the network (sbm_mlp_gradients,
+ * sbm_mlp_train, sbm_solve with the network attached) returns SBM_ERR_CUDA and clears the flag.  After
+ * that error of sbm_mlp_train the parameters are those of an unfinished epoch. */
 int sbm_mlp_gemm_backend(void* mlp, int backend);
 /* Polls after which a wait inside the one-launch kernel gives up: < 0 the default (2^22, also the
  * largest), 0 at once (for tests of the failure path).  A context takes the value at its first
