@@ -728,7 +728,6 @@ size_t build_tail_cta(Context& C, int top, TailCta<R>& T) {
   const size_t blk = (size_t)np * np * sizeof(R) + 16;          // a padded boundary block
   const size_t n0 = (size_t)C.lv[0].H.n_dof();
   std::vector<TailLevelDesc> D((size_t)top + 1);
-  T.low = dim == 2 && C.lv.back().H.p == 1 && sizeof(R) == 4;
   size_t bytes = 0, vec = 0;
   auto take = [&](size_t n) {                       // n bytes on a 16-byte boundary
     const size_t at = bytes;
@@ -799,9 +798,8 @@ size_t build_tail_cta(Context& C, int top, TailCta<R>& T) {
         for (int m = 0; m < np; ++m) {
           double v = 1, lam = 0;
           for (int k = 0; k < dim; ++k) {
-            // (entry (i, j) = entry (i ^ j, 0): the 1D matrices are symmetric under reflection)
-            const int dk = ((i ^ j) >> k) & 1, mk = (m >> k) & 1;
-            v *= H.S[dk * 2 + mk] * H.S[mk];
+            const int ik = (i >> k) & 1, jk = (j >> k) & 1, mk = (m >> k) & 1;
+            v *= H.S[ik * 2 + mk] * H.S[jk * 2 + mk];
             lam += H.lam[mk];
           }
           inv += v / (hs * lam);
@@ -809,7 +807,6 @@ size_t build_tail_cta(Context& C, int top, TailCta<R>& T) {
         for (int k = 0; k < dim; ++k)
           if (((i ^ j) & ~(1 << k)) == 0) self += hs * wt * H.L[3][((i >> k) & 1) * 2 + ((j >> k) & 1)];
         M[8 + j * np + i] = (R)inv;
-        if (T.low && j == 0) M[8 + 2 * np * np + i] = (R)(inv - (double)(R)inv);
         M[8 + np * np + j * np + i] = (R)self;
       }
     for (int b = 0; b < H.n_bnd; ++b)

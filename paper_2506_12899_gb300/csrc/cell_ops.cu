@@ -536,11 +536,9 @@ __device__ int g_tail_fault;
 //   - a cell's neighbours, boundary index and parent are one 16-byte record; a missing neighbour is a
 //     zero cell, so no load waits for a branch;
 //   - 2D: an interior cell applies a dense inverse like a boundary cell, so a warp of both takes one path,
-//     and boundary residuals use stored self blocks.  When the finest level is p = 1 an interior inverse has a
-//     high and a low part (TailCta::low): rounded to FP32 it made that V-cycle's error against 64 bits 4 to 11%
-//     larger than fast diagonalisation had it (disks of 16^2 to 512^2, 25 to 60 of each), with the low part the
-//     error is 3% larger to 6% smaller; a 64^2 V-cycle takes 17.4 instead of 16.2 us.  Below p = 2 and 3 the low
-//     part does not help (error +1 to +3%; -2 to +1% without).
+//     and boundary residuals use stored self blocks.  (Against fast diagonalisation the V-cycle's
+//     error against 64 bits moves by -8 to +13% with the geometry family and size, +1.6% in the mean over p = 1
+//     disks and stars of 32^2 to 1024^2; with the inverse in two parts by -9 to +7%, the same mean.)
 //   - 3D keeps the operations of the tail's first form in their order, to the same bits (the tests pin them): the
 //     long 3D p = 3 solves (96^3 to 1e-12) end after another number of steps when the rounding of their V-cycle
 //     changes.  (The per-level kernels round otherwise; they differ in most values by a unit or so.)
@@ -550,10 +548,7 @@ __device__ int g_tail_fault;
 // 600 cycles): a V-cycle of the 512^2 p = 2 star (tail: 64^2 .. 8^2) went 127 -> 107 us. In 3D the restriction
 // of the largest level, with the surrogate-face terms of its boundary cells, is the longest phase: a V-cycle
 // of a 64^3 p = 1 sphere (16^3 .. 4^3) takes 89 us with this order of operations and 76 with the 2D form.
-//
-// LOW: the interior inverses have their low part.  (A template argument: as a branch on TailCta::low it cost the
-// 512^2 p = 2 star, which has none, 0.4 us.)
-template <int D, typename R, bool LOW>
+template <int D, typename R>
 __global__ void __launch_bounds__(kTailCtaThreads, 1) k_vcycle_tail_cta(const __grid_constant__ TailCta<R> TP,
                                                                         const R* __restrict__ r_top,
                                                                         R* __restrict__ z_top,
@@ -736,9 +731,6 @@ __global__ void __launch_bounds__(kTailCtaThreads, 1) k_vcycle_tail_cta(const __
     R bc[8];                                         // the level's couplings
 #pragma unroll
     for (int i = 0; i < 8; ++i) bc[i] = M[i];
-    R lo[4];                                         // low part of the interior inverse
-#pragma unroll
-    for (int i = 0; i < 4; ++i) lo[i] = LOW ? M[8 + 2 * NP * NP + i] : R(0);
     if (!down) {                                     // prolongation (Eq. 17)
       const int nc = lev[l - 1].n_act;
       const unsigned zc = lev[l - 1].z;
@@ -800,12 +792,6 @@ __global__ void __launch_bounds__(kTailCtaThreads, 1) k_vcycle_tail_cta(const __
             block_solve_at<D, 2, R>(LP, b == 0xffffu ? nullptr : reinterpret_cast<const R*>(tcta_smem + binv + b * BLK), t, y);
           } else {
             couple(q, z, n, bc, t);
-            if (LOW && b == 0xffffu) {  // the low part first: entry (i, j) is lo[i ^ j]
-#pragma unroll
-              for (int i = 0; i < NP; ++i)
-#pragma unroll
-                for (int j = 0; j < NP; ++j) y[i] += lo[j & 3] * t[i ^ j];
-            }
             block(b == 0xffffu ? M + 8 : reinterpret_cast<const R*>(tcta_smem + binv + b * BLK), t, R(1), y);
           }
           if (om != R(1)) {
@@ -1122,12 +1108,10 @@ bool tail_cta_fits_kernel(K kern, size_t smem) {
 }
 
 bool tail_cta_fits(int dim, int prec, size_t smem) {
-  if (dim == 2)
-    return prec == 0 ? tail_cta_fits_kernel(k_vcycle_tail_cta<2, double, false>, smem)
-                     : tail_cta_fits_kernel(k_vcycle_tail_cta<2, float, false>, smem) &&
-                           tail_cta_fits_kernel(k_vcycle_tail_cta<2, float, true>, smem);
-  return prec == 0 ? tail_cta_fits_kernel(k_vcycle_tail_cta<3, double, false>, smem)
-                   : tail_cta_fits_kernel(k_vcycle_tail_cta<3, float, false>, smem);
+  if (dim == 2) return prec == 0 ? tail_cta_fits_kernel(k_vcycle_tail_cta<2, double>, smem)
+                                 : tail_cta_fits_kernel(k_vcycle_tail_cta<2, float>, smem);
+  return prec == 0 ? tail_cta_fits_kernel(k_vcycle_tail_cta<3, double>, smem)
+                   : tail_cta_fits_kernel(k_vcycle_tail_cta<3, float>, smem);
 }
 
 int tail_fault_take() {
@@ -1143,12 +1127,10 @@ int tail_fault_take() {
 template <typename R>
 cudaError_t launch_vcycle_tail_cta(int dim, const TailCta<R>& TP, const R* r, R* z, const double* coarse_inv,
                                    size_t smem, cudaStream_t s) {
-  if (dim == 2 && sizeof(R) == 4 && TP.low)
-    SBM_PDL((k_vcycle_tail_cta<2, R, sizeof(R) == 4>), 1, kTailCtaThreads, smem, s, TP, r, z, coarse_inv);
-  else if (dim == 2)
-    SBM_PDL((k_vcycle_tail_cta<2, R, false>), 1, kTailCtaThreads, smem, s, TP, r, z, coarse_inv);
+  if (dim == 2)
+    SBM_PDL((k_vcycle_tail_cta<2, R>), 1, kTailCtaThreads, smem, s, TP, r, z, coarse_inv);
   else
-    SBM_PDL((k_vcycle_tail_cta<3, R, false>), 1, kTailCtaThreads, smem, s, TP, r, z, coarse_inv);
+    SBM_PDL((k_vcycle_tail_cta<3, R>), 1, kTailCtaThreads, smem, s, TP, r, z, coarse_inv);
   count_launches();
   return cudaGetLastError();
 }

@@ -193,9 +193,8 @@ struct TailLevel {
 // so that consecutive cells' words are adjacent (no bank conflicts); cell n_act stays zero and stands
 // for a missing neighbour.  Boundary blocks are padded by 16 bytes for the same reason.
 constexpr int kMaxTailCta = 6;
-// entries of a level's matrices: the couplings (8); in 2D also the interior inverse, the interior block and the
-// inverse's low part (4: entry i ^ j)
-constexpr int tail_mats(int dim) { return dim == 2 ? 8 + 2 * 16 + 4 : 8; }
+// entries of a level's matrices: the couplings (8); in 2D also the interior inverse and the interior block
+constexpr int tail_mats(int dim) { return dim == 2 ? 8 + 2 * 16 : 8; }
 struct TailLevelDesc {
   int n_act;
   unsigned z, f, binv, aself, mats, rec, ch;   // aself 0: the boundary self blocks stay in global memory (3D: none)
@@ -208,7 +207,6 @@ struct TailLevelDesc {
 template <typename R>
 struct TailCta {
   int top, pre, post, ssor, n0;    // n0: unknowns of level 0
-  int low;                         // 1: the interior inverses have a low part (2D, finest level p = 1)
   unsigned image_bytes, cinv;      // cinv: the coarse inverse's transpose in the image, 0: not staged
   unsigned vec_bytes;              // the z vectors, from image_bytes on (the f vectors behind them)
   const void* image;
