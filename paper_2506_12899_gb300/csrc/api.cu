@@ -720,10 +720,11 @@ Context* build_context(const sbm_setup_desc& d, bool device) {
   return C.release();
 }
 
-// The one-CTA tail over levels 0..top: its parameters and, uploaded, its shared-memory image (TailCta).
+// The one-CTA tail over levels 0..top: its parameters and its shared-memory image (TailCta), copied to `room` on the
+// device.
 // Returns the bytes of shared memory, 0 if they do not fit (or an index does not fit its 16 bits).
 template <typename R>
-size_t build_tail_cta(Context& C, int top, TailCta<R>& T) {
+size_t build_tail_cta(Context& C, int top, void* room, TailCta<R>& T) {
   const int dim = C.lv[0].H.dim, np = C.lv[0].H.np, ncol = 1 << dim, pi = prec_index<R>();
   const size_t blk = (size_t)np * np * sizeof(R) + 16;          // a padded boundary block
   const size_t n0 = (size_t)C.lv[0].H.n_dof();
@@ -850,7 +851,8 @@ size_t build_tail_cta(Context& C, int top, TailCta<R>& T) {
   T.n0 = (int)n0;
   T.image_bytes = (unsigned)bytes;
   T.vec_bytes = (unsigned)vec;
-  T.image = C.upload(image);
+  CUDA_TRY(cudaMemcpy(room, image.data(), image.size(), cudaMemcpyHostToDevice));
+  T.image = room;
   T.T = tparams<R>(C.lv[1]);
   for (int l = 0; l <= top; ++l) T.P[l] = params<R>(C.lv[l]);
   return bytes + 2 * vec;
@@ -861,12 +863,19 @@ void ensure_work(Context& C) {
   const int pi = prec_index<R>();
   if (C.work_ready[pi]) return;
   for (auto& L : C.lv) ensure_blocks(C, L, R(0));
-  // one allocation for every level's vectors, each on a 256-byte boundary
+  // one allocation for every level's vectors, each on a 256-byte boundary, and for the one-CTA tail's image (at most
+  // an SM's shared memory) behind them
   const int nvec = C.desc.smoother == 0 ? 3 : (C.desc.smoother == 2 ? 5 : 4);
   auto padded = [](const DevLevel& L) { return ((size_t)L.H.n_dof() + 63) / 64 * 64; };
   size_t total = 0;
   for (auto& L : C.lv) total += nvec * padded(L);
-  R* next = C.dalloc<R>(total);
+  const bool tail_default = C.desc.tail_max_cells == 0;
+  const int ctas = C.desc.tail_cluster_ctas == 0 ? 1 : C.desc.tail_cluster_ctas;
+  // default (tail_max_cells = 0): the one-CTA tail for FP32 V-cycles, none for FP64 ones (one
+  // SM's FP64 pipe makes it slower than per-level launches: measured)
+  const bool one_cta = C.tail_cand >= 1 && ctas == 1 && !(tail_default && sizeof(R) == 8);
+  R* next = C.dalloc<R>(total + (one_cta ? (tail_smem_limit() + 1024) / sizeof(R) : 0));
+  void* const image_room = next + total;
   for (auto& L : C.lv) {
     void** slots[5] = {&L.z[pi], &L.rhs[pi], &L.res[pi], &L.tmp[pi], &L.dir[pi]};
     for (int k = 0; k < nvec; ++k, next += padded(L)) *slots[k] = next;
@@ -875,16 +884,12 @@ void ensure_work(Context& C) {
   // memory of a resident cluster of 16, else 8, CTAs
   C.tail_plan[pi] = TailPlan{};
   const int NP = C.lv[0].H.np;
-  // default (tail_max_cells = 0): the one-CTA tail for FP32 V-cycles, none for FP64 ones (one
-  // SM's FP64 pipe makes it slower than per-level launches: measured)
-  const bool tail_default = C.desc.tail_max_cells == 0;
-  const int ctas = C.desc.tail_cluster_ctas == 0 ? 1 : C.desc.tail_cluster_ctas;
-  if (ctas == 1 && !(tail_default && sizeof(R) == 8)) {
+  if (one_cta) {
     // one CTA: the highest candidate level whose data (levels 0..top) fit in its shared memory
     for (int top = std::min(C.tail_cand, kMaxTailCta - 1); top >= 1; --top) {
       auto tp = std::make_unique<TailCta<R>>();
       std::memset(static_cast<void*>(tp.get()), 0, sizeof(TailCta<R>));
-      const size_t smem = build_tail_cta<R>(C, top, *tp);
+      const size_t smem = build_tail_cta<R>(C, top, image_room, *tp);
       if (smem == 0) continue;
       C.tail_plan[pi].top = top;
       C.tail_plan[pi].cluster = 1;
